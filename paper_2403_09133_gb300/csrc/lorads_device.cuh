@@ -196,8 +196,14 @@ __device__ __forceinline__ T frag_dot_local(const Frag<T>& a, const Frag<T>& b) 
   return s;
 }
 
+// The lanes of a team arrive here from loads that only some of them make (a row's last chunks),
+// and their teams from loops of different lengths: they converge before they exchange.  Without
+// the __syncwarp the one-CTA FP64 kernel, depending on how it was compiled, exchanged across
+// lanes that had not met: matrix completion (r = 9, ld = 12: lane 1 of a team has no second
+// chunk) ran its first CG solve into the iteration limit, with other numbers in every run.
 template <typename T>
 __device__ __forceinline__ T team_sum(T x, const Team& t) {
+  __syncwarp(t.mask);
   for (int off = t.G >> 1; off > 0; off >>= 1) x += __shfl_xor_sync(t.mask, x, off);
   return x;
 }
