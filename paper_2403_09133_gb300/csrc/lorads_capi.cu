@@ -142,7 +142,7 @@ struct lorads_problem {
   void* dargs = nullptr;  // SolverArgs<T> on the device
   SolveOut* dout = nullptr;
   GridCtl* dctl = nullptr;
-  double* dpartials = nullptr;
+  Slot* dslots = nullptr;   // the barrier slots of a whole-GPU solve
   int* dqueue = nullptr;
   int sol_r = 0, sol_ld = 0;
   bool has_solution = false;
@@ -157,6 +157,13 @@ struct lorads_problem {
 // (LORADS_ERR_DEVICE): the caller's limit, else about a few seconds of polling
 static long long barrier_polls(const lorads_params* prm) {
   return prm->barrier_polls > 0 ? (long long)prm->barrier_polls : 50LL * 1000 * 1000;
+}
+
+// barrier slots of a whole-GPU solve: room for one copy of up to 8 CTAs per SM; a grid of nb CTAs
+// keeps as many copies as fit, at most SLOT_REPS
+static size_t grid_slot_doubles(int dev_sms) { return (size_t)dev_sms * 8 * SLOT_DOUBLES; }
+static int grid_slot_reps(int dev_sms, int nb) {
+  return std::max(1, std::min(SLOT_REPS, dev_sms * 8 / nb));
 }
 
 static bool is_finite_value(double x) { return std::isfinite(x); }
@@ -601,7 +608,7 @@ static int prepare_state(lorads_problem* p, const DevParams& dv, cudaStream_t s,
                  Arena::need(NS * ring, 8) * 2 +
                  Arena::need(1, sizeof(SolverArgs<T>)) + Arena::need(1, sizeof(SolveOut)) +
                  Arena::need(1, sizeof(GridCtl)) +
-                 Arena::need((size_t)dev_sms * 8 * MAXRED * 3, 8) + Arena::need(4, 4) + 4096;
+                 Arena::need(grid_slot_doubles(dev_sms), 8) + Arena::need(4, 4) + 4096;
   // the Lanczos vectors of a dual test: slots 0..Kmax of n x 4 doubles, when they fit the cap
   const int kmax = std::min(std::min(dv.lanczos_steps, LANCZOS_MAX), (int)std::min<int64_t>(n, INT32_MAX));
   const size_t store_count = dv.kkt_dinf && kmax > 0 ? (size_t)(kmax + 1) * (size_t)n * 4 : 0;
@@ -643,7 +650,7 @@ static int prepare_state(lorads_problem* p, const DevParams& dv, cudaStream_t s,
   p->dout = a.take<SolveOut>(1);
   h.out = p->dout;
   p->dctl = a.take<GridCtl>(1);
-  p->dpartials = a.take<double>((size_t)dev_sms * 8 * MAXRED * 3);
+  p->dslots = reinterpret_cast<Slot*>(a.take<double>(grid_slot_doubles(dev_sms)));
   p->dqueue = a.take<int>(4);
   p->dU = h.U;
   p->dV = h.V;
@@ -662,7 +669,7 @@ static int prepare_state(lorads_problem* p, const DevParams& dv, cudaStream_t s,
   unreached.status = ST_DEVICE;
   CU(cudaMemcpyAsync(p->dout, &unreached, sizeof(SolveOut), cudaMemcpyHostToDevice, s));
   CU(cudaMemsetAsync(p->dctl, 0, sizeof(GridCtl), s));
-  CU(cudaMemsetAsync(p->dpartials, 0xFF, sizeof(double) * (size_t)dev_sms * 8 * MAXRED * 3, s));
+  CU(cudaMemsetAsync(p->dslots, 0xFF, sizeof(double) * grid_slot_doubles(dev_sms), s));
   CU(cudaMemsetAsync(p->dqueue, 0, 16, s));
   *dargs_out = dargs;
   return LORADS_OK;
@@ -771,8 +778,9 @@ static int run_solve(lorads_problem* p, const lorads_params* prm, cudaStream_t s
   if (!whole) {
     le = Launch<T>::solve_block(dv.subsolver, dargs, 1, p->dqueue, 1, threads, s);
   } else {
-    le = Launch<T>::solve_grid(dv.subsolver, dargs, p->dctl, p->dpartials, barrier_polls(prm),
-                               grid, threads, s);
+    le = Launch<T>::solve_grid(dv.subsolver, dargs, p->dctl, p->dslots,
+                               grid_slot_reps(dev_sms, grid), barrier_polls(prm), grid, threads,
+                               s);
   }
   CU(le);
   SolveOut out{};
@@ -830,19 +838,19 @@ static int run_batch_once(lorads_problem* const* ps, int count, const lorads_par
     if (groups < 1) return LORADS_ERR_ARG;
     grid = groups * group;
   }
-  // argument block, queue, and for groups their barriers, problem slots and partial sums
+  // argument block, queue, and for groups their barriers, picked problems and barrier slots
   const size_t a_bytes = (sizeof(SolverArgs<T>) * count + 255) / 256 * 256;
   const size_t c_bytes = (sizeof(GridCtl) * groups + 255) / 256 * 256;
   const size_t s_bytes = (sizeof(int) * groups + 255) / 256 * 256;
-  const size_t p_bytes = sizeof(double) * (size_t)grid * MAXRED * (group > 1 ? 2 : 0);
+  const size_t p_bytes = group > 1 ? sizeof(double) * (size_t)grid * SLOT_DOUBLES : 0;
   const size_t base_bytes = a_bytes + 256 + c_bytes + s_bytes + p_bytes;
   char* base = static_cast<char*>(al.get(base_bytes));
   if (!base) return LORADS_ERR_NOMEM;
   SolverArgs<T>* dargs = reinterpret_cast<SolverArgs<T>*>(base);
   int* dqueue = reinterpret_cast<int*>(base + a_bytes);
   GridCtl* dctls = reinterpret_cast<GridCtl*>(base + a_bytes + 256);
-  int* dslots = reinterpret_cast<int*>(base + a_bytes + 256 + c_bytes);
-  double* dparts = reinterpret_cast<double*>(base + a_bytes + 256 + c_bytes + s_bytes);
+  int* dpicks = reinterpret_cast<int*>(base + a_bytes + 256 + c_bytes);
+  Slot* dslots = reinterpret_cast<Slot*>(base + a_bytes + 256 + c_bytes + s_bytes);
   int st = LORADS_OK;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaStream_t cap = nullptr;
@@ -860,8 +868,9 @@ static int run_batch_once(lorads_problem* const* ps, int count, const lorads_par
         LORADS_OK) break;
     cudaError_t c1 = cudaMemsetAsync(dqueue, 0, 16, cap);
     if (c1 == cudaSuccess && group > 1) c1 = cudaMemsetAsync(dctls, 0, c_bytes, cap);
+    if (c1 == cudaSuccess && group > 1) c1 = cudaMemsetAsync(dslots, 0xFF, p_bytes, cap);
     const cudaError_t c2 =
-        group > 1 ? Launch<T>::solve_group(sub, dargs, count, dqueue, dctls, dparts, dslots, group,
+        group > 1 ? Launch<T>::solve_group(sub, dargs, count, dqueue, dctls, dslots, dpicks, group,
                                            barrier_polls(prm), grid, threads, cap)
                   : Launch<T>::solve_block(sub, dargs, count, dqueue, grid, threads, cap);
     const cudaError_t c3 = cudaStreamEndCapture(cap, &graph);
@@ -1469,11 +1478,11 @@ static int run_solve_static(lorads_problem* p, const lorads_params* prm, cudaStr
   SolverArgs<T>* dargs = a.take<SolverArgs<T>>(1);
   SolveOut* dout = a.take<SolveOut>(1);
   GridCtl* dctl = a.take<GridCtl>(1);
-  double* dpartials = a.take<double>((size_t)dev_sms * 8 * MAXRED * 3);
+  Slot* dslots = reinterpret_cast<Slot*>(a.take<double>(grid_slot_doubles(dev_sms)));
   int* dqueue = a.take<int>(4);
   if (!h.U || !h.V || !h.Ut || !h.Vt || !h.Dl || !h.R || !h.Pd || !h.HP || !h.Sv || !h.lam ||
       !h.e || !h.cq || !h.grad || !h.grad_old || !h.dir || !h.tmp || !h.CWn || !h.S || !h.Y ||
-      !dargs || !dout || !dctl || !dpartials || !dqueue)
+      !dargs || !dout || !dctl || !dslots || !dqueue)
     return LORADS_ERR_TOO_LARGE;
   h.out = dout;
   if (!dv.phase1) {
@@ -1486,14 +1495,14 @@ static int run_solve_static(lorads_problem* p, const lorads_params* prm, cudaStr
   unreached.status = ST_DEVICE;
   CU(cudaMemcpyAsync(dout, &unreached, sizeof(SolveOut), cudaMemcpyHostToDevice, s));
   CU(cudaMemsetAsync(dctl, 0, sizeof(GridCtl), s));
-  CU(cudaMemsetAsync(dpartials, 0xFF, sizeof(double) * (size_t)dev_sms * 8 * MAXRED * 3, s));
+  CU(cudaMemsetAsync(dslots, 0xFF, sizeof(double) * grid_slot_doubles(dev_sms), s));
   CU(cudaMemsetAsync(dqueue, 0, 16, s));
   cudaError_t le;
   if (!whole) {
     le = Launch<T>::solve_block(dv.subsolver, dargs, 1, dqueue, 1, threads, s);
   } else {
-    le = Launch<T>::solve_grid(dv.subsolver, dargs, dctl, dpartials, barrier_polls(prm), grid,
-                               threads, s);
+    le = Launch<T>::solve_grid(dv.subsolver, dargs, dctl, dslots, grid_slot_reps(dev_sms, grid),
+                               barrier_polls(prm), grid, threads, s);
   }
   CU(le);
   SolveOut out{};

@@ -14,6 +14,11 @@
 //     constraint id, for the sparse-times-dense products.  Constraints with several entries
 //     are also cut into chunks of at most CON_CHUNK entries (chunk_ptr; con_chunk gives each
 //     constraint's chunks) so that a long constraint is summed by many teams.
+//   * Shuffles always name the whole warp, so every loop over teams runs the same number of
+//     rounds in all lanes of a warp (TeamRows): teams past the end take part with empty rows.
+//     A shuffle that names only its team's lanes splits the warp: one 8-element dot product with
+//     its team sum took 478 clocks in teams of 2 and 552 in teams of 4 (9 warps per SM), 126 and
+//     169 with the whole warp named.
 //   * Reductions are deterministic: fixed shuffle trees inside warps, warps summed in order,
 //     CTAs summed in order by the last CTA to arrive at the grid barrier.
 #pragma once
@@ -24,6 +29,7 @@ namespace lorads {
 
 constexpr int KMAX = 2;      // chunks per lane
 constexpr int CHUNK = 4;     // elements per chunk (16 B of float, 32 B of double)
+constexpr int RED_ROWS = 36;  // rows of a scope's shared array (see BlockScope)
 constexpr int MAXRED = 12;   // values per reduction (the last slot carries the barrier status)
 constexpr int MAXMEM = 8;    // L-BFGS memory cap
 constexpr int CON_CHUNK = 32;  // entries per chunk of a multi-entry constraint
@@ -91,8 +97,11 @@ struct Team {
   int lane;       // lane inside the team
   int id;         // team index inside the scope
   int count;      // teams in the scope
-  int nc;         // chunks per row (ld / 4)
-  unsigned mask;  // shuffle mask of the team's lanes
+  int nc;         // chunks per row (ld / 4); 0 for a team past the end of its loop
+  int sub;        // team index inside the warp
+  int first;      // index of the warp's first team
+  bool live;      // false for a team past the end of its loop
+  bool lead;      // the first lane of a live team
 };
 
 __host__ __device__ inline int team_size_for(int ld) {
@@ -111,11 +120,37 @@ __device__ inline Team make_team(int ld, int tid, int nthreads, int mult = 1) {
   t.id = tid / t.G;
   t.count = nthreads / t.G;
   t.nc = ld / CHUNK;
-  int wl = threadIdx.x & 31;
-  int base = wl & ~(t.G - 1);
-  t.mask = (t.G == 32) ? 0xffffffffu : (((1u << t.G) - 1u) << base);
+  t.sub = (threadIdx.x & 31) / t.G;
+  t.first = t.id - t.sub;
+  t.live = true;
+  t.lead = t.lane == 0;
   return t;
 }
+
+// A loop of the teams over rows 0 .. n-1 (row j to team j mod count) in which the lanes of a warp
+// stay together: a team whose row lies past the end takes the last round with live = false, an
+// empty row (nc = 0: loads give zeros, stores store nothing) and j clamped into range.
+struct TeamRows {
+  Team t;
+  int j;
+  int base, n, nc;
+  __device__ __forceinline__ TeamRows(const Team& tm, int rows)
+      : t(tm), base(tm.first), n(rows), nc(tm.nc) {
+    place();
+  }
+  __device__ __forceinline__ bool more() const { return base < n; }
+  __device__ __forceinline__ void next() {
+    base += t.count;
+    place();
+  }
+  __device__ __forceinline__ void place() {
+    j = base + t.sub;
+    t.live = j < n;
+    t.nc = t.live ? nc : 0;
+    t.lead = t.live && t.lane == 0;
+    if (!t.live) j = n - 1;
+  }
+};
 
 template <typename T>
 struct Frag {
@@ -196,15 +231,14 @@ __device__ __forceinline__ T frag_dot_local(const Frag<T>& a, const Frag<T>& b) 
   return s;
 }
 
-// The lanes of a team arrive here from loads that only some of them make (a row's last chunks),
-// and their teams from loops of different lengths: they converge before they exchange.  Without
-// the __syncwarp the one-CTA FP64 kernel, depending on how it was compiled, exchanged across
-// lanes that had not met: matrix completion (r = 9, ld = 12: lane 1 of a team has no second
-// chunk) ran its first CG solve into the iteration limit, with other numbers in every run.
+// Sum over the lanes of each team, called by whole warps.  The lanes arrive here from loads that
+// only some of them make (a row's last chunks) and converge before they exchange: without that
+// the one-CTA FP64 kernel, depending on how it was compiled, exchanged across lanes that had not
+// met (matrix completion, r = 9, ld = 12: lane 1 of a team has no second chunk).
 template <typename T>
 __device__ __forceinline__ T team_sum(T x, const Team& t) {
-  __syncwarp(t.mask);
-  for (int off = t.G >> 1; off > 0; off >>= 1) x += __shfl_xor_sync(t.mask, x, off);
+  __syncwarp();
+  for (int off = t.G >> 1; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
   return x;
 }
 
@@ -252,31 +286,14 @@ __device__ inline double normal_at(uint64_t key, uint64_t e) {
 // ------------------------------------------------------------------------------------
 // scopes: one CTA, or the whole grid of a cooperative launch
 // ------------------------------------------------------------------------------------
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
 __device__ __forceinline__ int ld_acquire_s32(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ unsigned atom_add_acq_rel_u32(unsigned* p, unsigned v) {
-  unsigned old;
-  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-  return old;
-}
-__device__ __forceinline__ void red_add_release_u32(unsigned* p, unsigned v) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 struct GridCtl {
-  unsigned int count;
-  unsigned int gen;
-  int error;
-  int pad;
-  double result[MAXRED];
+  int error;      // a barrier gave up: every CTA of the scope leaves at its next wait
+  int pad[3];
 };
 
 // Sum over the 32 lanes of a warp of K values (K a power of two, <= 16) by recursive halving:
@@ -313,67 +330,76 @@ __device__ __forceinline__ bool scatter_writer() {
   return ((threadIdx.x & 31) & (32 / K - 1)) == 0;
 }
 
+// Stage 1 of a reduction: the warp sums of k values into red[warp * MAXRED + i].
 template <int K>
-__device__ __forceinline__ void block_reduce_k(double* v, int k, double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+__device__ __forceinline__ void warp_sums_k(const double* v, int k, double* red) {
+  const int warp = threadIdx.x >> 5;
   double w[K];
 #pragma unroll
   for (int i = 0; i < K; ++i) w[i] = i < k ? v[i] : 0.0;
-  int ix = warp_sum_scatter<K>(w);
+  const int ix = warp_sum_scatter<K>(w);
   if (scatter_writer<K>() && ix < k) red[warp * MAXRED + ix] = w[0];
-  __syncthreads();
-  if (warp == 0) {
+}
+__device__ __forceinline__ void warp_sums(const double* v, int k, double* red) {
+  __syncwarp();
+  if (k <= 1) warp_sums_k<1>(v, k, red);
+  else if (k <= 2) warp_sums_k<2>(v, k, red);
+  else if (k <= 4) warp_sums_k<4>(v, k, red);
+  else if (k <= 8) warp_sums_k<8>(v, k, red);
+  else warp_sums_k<16>(v, k, red);
+}
+// Stage 1 for two values carried by teams of G lanes.  G >= 2: value 0 sits in the teams' even
+// lanes' x0 and value 1 in their odd lanes' x0, so one butterfly over the lane offsets 16 .. G
+// sums both (offsets below G would only add a team's lanes to one another); G = 1: every lane
+// carries both.  The additions of each value are those of warp_sum_scatter with the values in
+// lane 0 of each team.
+__device__ __forceinline__ void warp_sums_pair(double x0, double x1, int G, double* red) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncwarp();
+  if (G >= 2) {
+    for (int off = 16; off >= G; off >>= 1) x0 += __shfl_xor_sync(0xffffffffu, x0, off);
+    if (lane < 2) red[warp * MAXRED + lane] = x0;
+  } else {
+    const double v[2] = {x0, x1};
+    warp_sums_k<2>(v, 2, red);
+  }
+}
+
+// Stage 2, by one warp: the sum of value i over the CTA's warps (at most 16) in the order of a
+// butterfly, in every lane below 16.
+__device__ __forceinline__ double block_sum(int i, const double* red) {
+  const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+  double x = lane < nw ? red[lane * MAXRED + i] : 0.0;
 #pragma unroll
-    for (int i = 0; i < K; ++i) w[i] = (lane < nw && i < k) ? red[lane * MAXRED + i] : 0.0;
-    ix = warp_sum_scatter<K>(w);
-    if (scatter_writer<K>() && ix < k) red[32 * MAXRED + ix] = w[0];
+  for (int off = 8; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  return x;
+}
+
+// deterministic CTA-wide sum of k (< MAXRED) values; every thread receives the sums in v.
+// Warp i finishes value i, so the second stage takes one chain of four additions whatever k is.
+__device__ inline void block_reduce(double* v, int k, double* red /* smem [33*MAXRED] */) {
+  const int nw = (blockDim.x + 31) >> 5;
+  warp_sums(v, k, red);
+  __syncthreads();
+  for (int i = threadIdx.x >> 5; i < k; i += nw) {
+    const double x = block_sum(i, red);
+    if ((threadIdx.x & 31) == 0) red[32 * MAXRED + i] = x;
   }
   __syncthreads();
   for (int i = 0; i < k; ++i) v[i] = red[32 * MAXRED + i];
 }
 
-// deterministic CTA-wide sum of k (< MAXRED) values; every thread receives the sums in v
-__device__ inline void block_reduce(double* v, int k, double* red /* smem [33*MAXRED] */) {
-  if (k <= 1) block_reduce_k<1>(v, k, red);
-  else if (k <= 2) block_reduce_k<2>(v, k, red);
-  else if (k <= 4) block_reduce_k<4>(v, k, red);
-  else if (k <= 8) block_reduce_k<8>(v, k, red);
-  else block_reduce_k<16>(v, k, red);
-}
-
-// Warp 0 of a CTA: the sum over nb CTAs of the k partials each left in partials[b * MAXRED + i],
-// into red[32 * MAXRED + i].  Lane l adds the CTAs l, l + 32, ...; the loads of a lane are
-// issued together (32 / K CTAs per round trip), then the lanes combine by warp_sum_scatter.
-template <int K>
-__device__ __forceinline__ void grid_partials_k(const double* partials, int k, int nb,
-                                                double* red) {
-  constexpr int TC = 32 / K;
-  const int lane = threadIdx.x & 31;
-  double w[K];
-#pragma unroll
-  for (int i = 0; i < K; ++i) w[i] = 0.0;
-  for (int b0 = 0; b0 < nb; b0 += 32 * TC) {
-    double buf[TC][K];
-#pragma unroll
-    for (int t = 0; t < TC; ++t) {
-      const int b = b0 + lane + 32 * t;
-#pragma unroll
-      for (int i = 0; i < K; ++i)
-        buf[t][i] = (b < nb && i < k) ? __ldcg(partials + b * MAXRED + i) : 0.0;
-    }
-#pragma unroll
-    for (int t = 0; t < TC; ++t)
-#pragma unroll
-      for (int i = 0; i < K; ++i) w[i] += buf[t][i];
-  }
-  const int ix = warp_sum_scatter<K>(w);
-  if (scatter_writer<K>() && ix < k) red[32 * MAXRED + ix] = w[0];
-}
-
-// Scopes: the CTA's shared array `red` holds 34 rows of MAXRED doubles: rows 0..31 the
-// per-warp sums of a reduction, row 32 its results, row 33 per-CTA scalar scratch for the
+// Scopes: the CTA's shared array `red` holds RED_ROWS rows of MAXRED doubles: rows 0..31 the
+// per-warp sums of a reduction, row 32 its results, rows 33..35 per-CTA scalar scratch for the
 // solver (no __shared__ variables are declared inside solver functions, which several kernels
 // instantiate).
+//
+// reduce_pair sums two values given in warp_sums_pair's form and calls f(sum 0, sum 1) in thread 0
+// of every CTA before the CTA goes on: f evaluates the scalars that follow from the sums (FP64
+// divides issue at 1/64 of the FP32 rate here, so one thread per CTA does it) and leaves them in
+// the scratch row.  reduce_each(v, k, f) calls f(i, sum i) for each value in one thread of the
+// CTA.  EXCHANGE tells whether the scope's CTAs also read one another's memory writes after it;
+// without, a reduction orders nothing but its sums.
 struct BlockScope {
   double* red;
   __device__ double* scratch() const { return red + 33 * MAXRED; }
@@ -387,17 +413,134 @@ struct BlockScope {
     block_reduce(v, k, red);
     return true;
   }
+  template <bool EXCHANGE, class F>
+  __device__ __forceinline__ bool reduce_pair(double x0, double x1, int G, F f) {
+    warp_sums_pair(x0, x1, G, red);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      // lanes 0-15 finish value 0, lanes 16-31 value 1 (block_sum's order)
+      const int lane = threadIdx.x, w = lane & 15, nw = (blockDim.x + 31) >> 5;
+      double x = w < nw ? red[w * MAXRED + (lane >> 4)] : 0.0;
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+      const double o = __shfl_sync(0xffffffffu, x, 16);
+      if (lane == 0) f(x, o);
+    }
+    __syncthreads();
+    return true;
+  }
+  template <class F>
+  __device__ __forceinline__ bool reduce_each(const double* v, int k, F f) {
+    const int nw = (blockDim.x + 31) >> 5;
+    warp_sums(v, k, red);
+    __syncthreads();
+    for (int i = threadIdx.x >> 5; i < k; i += nw) {
+      const double x = block_sum(i, red);
+      if ((threadIdx.x & 31) == 0) f(i, x);
+    }
+    __syncthreads();
+    return true;
+  }
   __device__ bool is_leader() const { return threadIdx.x == 0; }
 };
 
+// a CTA's partial sum of one value and the number of the barrier it belongs to, stored and
+// loaded as one 128-bit access (single-copy atomic as a relaxed .b128 access)
+struct alignas(16) Slot {
+  double v;
+  unsigned long long tag;
+};
+__device__ __forceinline__ void st_slot(Slot* p, double v, unsigned long long tag) {
+  asm volatile(
+      "{\n .reg .b128 q;\n mov.b128 q, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], q;\n}\n" ::"l"(p),
+      "l"(__double_as_longlong(v)), "l"(tag)
+      : "memory");
+}
+__device__ __forceinline__ void ld_slot(const Slot* p, double& v, unsigned long long& tag) {
+  long long a;
+  unsigned long long b;
+  asm volatile(
+      "{\n .reg .b128 q;\n ld.relaxed.gpu.global.b128 q, [%2];\n mov.b128 {%0, %1}, q;\n}\n"
+      : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  v = __longlong_as_double(a);
+  tag = b;
+}
+__device__ __forceinline__ void fence_release_gpu() {
+  asm volatile("fence.release.gpu;" ::: "memory");
+}
+__device__ __forceinline__ void fence_acquire_gpu() {
+  asm volatile("fence.acquire.gpu;" ::: "memory");
+}
+
+// One warp: polls the slots of c CTAs until every tag is `bar` and returns the sum of their values:
+// lane l adds the CTAs l, l + 32, ... and the lanes combine by a butterfly.  ok turns false when
+// the wait is given up: after `limit` polls (which sets *error) or when *error is set.  A function
+// of its own: inlined at every reduction its buffers pushed the solver's rows out of registers.
+static __device__ __noinline__ double poll_slots(const Slot* from, int c, unsigned bar, int* error,
+                                          long long limit, bool& ok) {
+  constexpr int TC = 5;            // 160 CTAs per round of loads
+  const int lane = threadIdx.x & 31;
+  double s = 0.0;
+  long long it = 0;
+  bool good = true;
+  for (int b0 = 0; b0 < c && good; b0 += 32 * TC) {
+    double v[TC];
+    for (;;) {
+      bool all = true;
+#pragma unroll
+      for (int t = 0; t < TC; ++t) {
+        const int b = b0 + lane + 32 * t;
+        unsigned long long tag = bar;
+        v[t] = 0.0;
+        if (b < c) ld_slot(from + b, v[t], tag);
+        all = all && tag == bar;
+      }
+      if (all) break;
+      if ((++it & 63) == 0 && ld_acquire_s32(error)) good = false;
+      if (good && it > limit) {
+        atomicExch(error, 1);
+        good = false;
+      }
+      if (!good) break;
+    }
+#pragma unroll
+    for (int t = 0; t < TC; ++t) s = (b0 == 0 && t == 0) ? v[0] : s + v[t];
+  }
+  ok = __all_sync(0xffffffffu, good);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  return s;
+}
+
+constexpr int SLOT_VALUES = 9;    // values of one reduction, at most
+constexpr int SLOT_REPS = 4;      // copies of every slot, at most (at most 16: one lane stores each)
+// doubles of slot memory per CTA of a scope and copy: two barriers x SLOT_VALUES x 16 bytes
+constexpr int SLOT_DOUBLES = 2 * SLOT_VALUES * 2;
+
+// A scope of several co-resident CTAs.  A reduction leaves each CTA's sum of every value in a
+// slot of its own, tagged with the barrier's number; a CTA polls the slots of all CTAs until
+// the tags match and adds the values in CTA order: lane l of a value takes the CTAs l, l + 32, ...
+// and the lanes combine by a butterfly, so every CTA forms the same sums.  There is no counter:
+// on the critical path are one store's way to L2 and one load's way back, where an arrival on a
+// counter, its release, the wait for it and the loads of the partial sums are four such ways.
+// Slots are kept in `reps` copies, CTA b polling copy b % reps: one copy polled by 152 CTAs is
+// a hot spot that delays the stores behind it.  Measured at 152 x 288 threads, two values,
+// memory writes ordered: 5.08 us with a counter, 5.48 / 4.37 / 3.90 / 3.95 / 4.40 / 4.49 us with 1 / 2 /
+// 4 / 8 / 16 / 152 copies; 3.32 us (4 copies) when only the sums are exchanged, since the release
+// fence is not needed.
+// Consecutive barriers use two sets of slots by the parity of their number: a CTA stores for
+// barrier g + 2 only after it passed g + 1, where every CTA had stored, that is, had finished
+// reading barrier g.  Tags start at 1 and the slots hold no valid tag at launch (the host fills
+// them with 0xFF), so stale contents never match.
 struct GridScope {
-  double* red;             // shared memory (34 rows of MAXRED, see BlockScope)
+  double* red;             // shared memory (see BlockScope)
   GridCtl* ctl;            // zeroed before launch
-  double* partials;        // 2 * gridDim.x * MAXRED (two rounds, by barrier generation)
+  Slot* slots;             // reps copies of 2 x SLOT_VALUES x count() slots
+  int reps;
   long long spin_limit;    // polls before a barrier gives up
   int first = 0;           // the scope spans CTAs [first, first + nb) of a cooperative launch
   int nb = 0;              // (0: the whole grid)
-  unsigned gen_next = 0;   // thread 0: the generation of its next barrier (ctl->gen starts at 0)
+  unsigned gen = 0;        // number of the last barrier
 
   __device__ int count() const { return nb > 0 ? nb : (int)gridDim.x; }
   __device__ double* scratch() const { return red + 33 * MAXRED; }
@@ -405,80 +548,77 @@ struct GridScope {
   __device__ int nthreads() const { return count() * blockDim.x; }
   __device__ bool is_leader() const { return (int)blockIdx.x == first && threadIdx.x == 0; }
 
-  // Bounded barrier over the scope's CTAs.  With k > 0 it also sums, over CTAs in CTA order, the
-  // CTA sums left in red[32*MAXRED + i] by block_reduce.  Arrival is an acq_rel increment of
-  // ctl->count; the last CTA resets the count and releases the generation; the others poll
-  // the generation with acquire loads (bounded).  Every CTA then loads all partials -- the
-  // loads of one lane are issued together, eight CTAs at a time, so their L2 round trips
-  // overlap -- and adds them in the same fixed order.
-  // The partials of consecutive barriers go to two buffers chosen by the parity of the
-  // barrier's generation: a CTA released early may reach the next reduction and store its
-  // next partial while a later CTA still loads this round's, so one buffer would let the later
-  // CTA add a value of the wrong round.  Two rounds suffice, since no CTA passes the next
-  // barrier before every CTA has arrived there, that is, has finished reading this round.
-  // Thread 0 knows the generation in advance (the one it saw released, plus one), so nothing
-  // is loaded before the arrival: on the critical path are the arrival's atomic, the release's
-  // visibility to the waiters and the load of the partials.  (Loading the generation first, as
-  // a check, cost one more L2 round trip per barrier.  Per-CTA release flags that every CTA
-  // polls, with no atomic, were slower: 152 CTAs polling 152 lines.)
-  __device__ bool barrier(int k) {
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
-      int ok = 1;
-      unsigned parity = 0;
-      if (lane == 0) {
-        parity = gen_next & 1u;
-        double* mine = partials + (size_t)parity * gridDim.x * MAXRED;
-        for (int i = 0; i < k; ++i) mine[blockIdx.x * MAXRED + i] = red[32 * MAXRED + i];
-        const unsigned my_gen = gen_next;
-        gen_next = my_gen + 1u;
-        const unsigned arrived = atom_add_acq_rel_u32(&ctl->count, 1u);
-        if (arrived == (unsigned)count() - 1) {
-          ctl->count = 0;
-          red_add_release_u32(&ctl->gen, 1u);
-        } else {
-          long long it = 0;
-          while (ld_acquire_u32(&ctl->gen) == my_gen) {
-            if ((++it & 63) == 0 && ld_acquire_s32(&ctl->error)) {
-              ok = 0;
-              break;
-            }
-            if (it > spin_limit) {
-              atomicExch(&ctl->error, 1);
-              ok = 0;
-              break;
-            }
-            __nanosleep(32);
-          }
-        }
-        red[32 * MAXRED + MAXRED - 1] = ok ? 0.0 : 1.0;
-      }
-      // lane 0's acquire orders the other lanes' loads through __syncwarp
-      __syncwarp();
-      parity = __shfl_sync(0xffffffffu, parity, 0);
-      if (k > 0) {
-        const int c = count();
-        const double* pp = partials + ((size_t)parity * gridDim.x + first) * MAXRED;
-        if (k <= 1) grid_partials_k<1>(pp, k, c, red);
-        else if (k <= 2) grid_partials_k<2>(pp, k, c, red);
-        else if (k <= 4) grid_partials_k<4>(pp, k, c, red);
-        else if (k <= 8) grid_partials_k<8>(pp, k, c, red);
-        else grid_partials_k<16>(pp, k, c, red);
-      }
-    }
+  // clears the failure mark; every thread, once, before the scope's first barrier
+  __device__ void init() {
+    if (threadIdx.x == 0) red[32 * MAXRED + MAXRED - 1] = 0.0;
     __syncthreads();
-    return red[32 * MAXRED + MAXRED - 1] == 0.0;
+  }
+  __device__ bool failed() const { return red[32 * MAXRED + MAXRED - 1] != 0.0; }
+
+  // One warp: stores the CTA's sum x of value i (the same in every lane below 16) and returns the
+  // sum over the scope in every lane.  `bar` is the barrier's number.
+  template <bool EXCHANGE>
+  __device__ __forceinline__ double exchange(double x, int i, unsigned bar) {
+    const int lane = threadIdx.x & 31, c = count(), me = (int)blockIdx.x - first;
+    const size_t copy = (size_t)2 * SLOT_VALUES * c;
+    Slot* set = slots + ((size_t)(bar & 1u) * SLOT_VALUES + i) * c;
+    if (EXCHANGE) fence_release_gpu();
+    if (lane < reps) st_slot(set + lane * copy + me, x, bar);
+    bool ok = true;
+    const double s = poll_slots(set + (me % reps) * copy, c, bar, &ctl->error, spin_limit, ok);
+    if (EXCHANGE) fence_acquire_gpu();
+    if (!ok) red[32 * MAXRED + MAXRED - 1] = 1.0;
+    return s;
   }
 
   __device__ bool sync() {
+    const unsigned bar = ++gen;
     __syncthreads();
-    return barrier(0);
+    if (threadIdx.x < 32) exchange<true>(0.0, 0, bar);
+    __syncthreads();
+    return !failed();
+  }
+
+  // f(i, sum i) in lane 0 of the warp that finishes value i
+  template <class F>
+  __device__ __forceinline__ bool reduce_each(const double* v, int k, F f) {
+    const int nw = (blockDim.x + 31) >> 5;
+    warp_sums(v, k, red);
+    const unsigned bar = ++gen;
+    __syncthreads();
+    for (int i = threadIdx.x >> 5; i < k; i += nw) {
+      const double s = exchange<true>(block_sum(i, red), i, bar);
+      if ((threadIdx.x & 31) == 0) f(i, s);
+    }
+    __syncthreads();
+    return !failed();
   }
   __device__ bool reduce(double* v, int k) {
-    block_reduce(v, k, red);   // leaves CTA sums in red[32*MAXRED + i]
-    bool ok = barrier(k);
-    for (int i = 0; i < k; ++i) v[i] = red[32 * MAXRED + i];
+    double* out = red + 32 * MAXRED;
+    const bool ok = reduce_each(v, k, [out](int i, double s) { out[i] = s; });
+    for (int i = 0; i < k; ++i) v[i] = out[i];
     return ok;
+  }
+  template <bool EXCHANGE, class F>
+  __device__ __forceinline__ bool reduce_pair(double x0, double x1, int G, F f) {
+    warp_sums_pair(x0, x1, G, red);
+    const unsigned bar = ++gen;
+    __syncthreads();
+    const int warp = threadIdx.x >> 5;
+    if (warp < 2) {
+      const double s = exchange<EXCHANGE>(block_sum(warp, red), warp, bar);
+      // warp 1 hands its sum to warp 0 (a named barrier of the two)
+      if (warp == 1) {
+        if (threadIdx.x == 32) red[32 * MAXRED] = s;
+        __syncwarp();
+        asm volatile("bar.arrive 1, 64;" ::: "memory");
+      } else {
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+        if (threadIdx.x == 0) f(s, red[32 * MAXRED]);
+      }
+    }
+    __syncthreads();
+    return !failed();
   }
 };
 
@@ -494,34 +634,18 @@ struct GroupScope : GridScope {};
 // Hessian of eq. linU on row j with fixed factor W:
 //   (H P)_j = rho * sum_{entries (j,k) of A_i} a q_i W_k + gamma P_j,
 //   q_i = <A_i, P W^T> = a (P_j . W_k + P_k . W_j)   (off-diagonal)   or   a P_j . W_j.
-// Returns the row in out; Pj is loaded by the caller (it is also needed for p.Hp).
+// This form: every constraint is one diagonal entry, at most one per row (a: row j's value, 0
+// without a constraint).  Returns the row in out; called by whole warps.
 template <typename T>
-__device__ __forceinline__ void hessian_row(const DevProblem& P, const T* Wm, const T* Pm,
-                                            int ld, int j, const Frag<T>& Pj, T rho, T gamma,
-                                            const Team& t, Frag<T>& out) {
-  Frag<T> Wj, acc;
-  frag_load(Wj, Wm, j, ld, t);
-  frag_zero(acc);
-  const T* av = aval<T>(P);
-  const int e0 = P.A_rp[j], e1 = P.A_rp[j + 1];
-  for (int e = e0; e < e1; ++e) {
-    const int k = P.A_col[e];
-    const T a = av[e];
-    if (k == j) {
-      T q = a * frag_dot(Pj, Wj, t);
-      frag_axpy(acc, a * q, Wj);
-    } else {
-      Frag<T> Wk, Pk;
-      frag_load(Wk, Wm, k, ld, t);
-      frag_load(Pk, Pm, k, ld, t);
-      T q = a * team_sum(frag_dot_local(Pj, Wk) + frag_dot_local(Pk, Wj), t);
-      frag_axpy(acc, a * q, Wk);
-    }
-  }
+__device__ __forceinline__ void hessian_row(T a, const Frag<T>& Wj, const Frag<T>& Pj, T rho,
+                                            T gamma, const Team& t, Frag<T>& out) {
+  const T q = a * frag_dot(Pj, Wj, t);
+  const T aq = a * q;
 #pragma unroll
   for (int kk = 0; kk < KMAX; ++kk)
 #pragma unroll
-    for (int ee = 0; ee < CHUNK; ++ee) out.v[kk][ee] = fma(rho, acc.v[kk][ee], gamma * Pj.v[kk][ee]);
+    for (int ee = 0; ee < CHUNK; ++ee)
+      out.v[kk][ee] = fma(rho, aq * Wj.v[kk][ee], gamma * Pj.v[kk][ee]);
 }
 
 // (A^T(w) - C) W on row j, w_i = wb * b_i + wl * lambda_i + we * e_i (e may be NULL),
@@ -593,34 +717,21 @@ __device__ __forceinline__ double sddmm_entry(const T* Um, const T* Vm, int ld, 
   return a * (double)team_sum(loc, t);
 }
 
-// <A_i, U V^T>: the sum over constraint i's entries (team-cooperative)
+// <A_i, U V^T>: the sum over constraint i's entries (team-cooperative; called by whole warps, whose
+// teams take as many rounds as the longest of their constraints)
 template <typename T>
 __device__ __forceinline__ double sddmm_con(const DevProblem& P, const T* Um, const T* Vm, int ld,
                                             int i, const Team& t) {
+  const int e0 = P.con_ptr[i], cnt = t.live ? P.con_ptr[i + 1] - e0 : 0;
+  const int rounds = P.a_multi ? __reduce_max_sync(0xffffffffu, cnt) : 1;
   double s = 0.0;
-  for (int e = P.con_ptr[i]; e < P.con_ptr[i + 1]; ++e)
-    s += sddmm_entry<T>(Um, Vm, ld, P.con_r[e], P.con_c[e], P.con_a[e], t);
-  return s;
-}
-
-// Hessian row of eq. linU for multi-entry constraints, from q_i = <A_i, P W^T> computed
-// beforehand: (H P)_j = rho sum_{entries (j,k) of A_i} a q_i W_k + gamma P_j (one team)
-template <typename T>
-__device__ __forceinline__ void hessian_row_q(const DevProblem& P, const T* Wm, int ld, int j,
-                                              const Frag<T>& Pj, const double* q, T rho, T gamma,
-                                              const Team& t, Frag<T>& out) {
-  Frag<T> acc;
-  frag_zero(acc);
-  const T* av = aval<T>(P);
-  for (int e = P.A_rp[j]; e < P.A_rp[j + 1]; ++e) {
-    Frag<T> Wk;
-    frag_load(Wk, Wm, P.A_col[e], ld, t);
-    frag_axpy(acc, av[e] * (T)q[P.A_con[e]], Wk);
+  for (int k = 0; k < rounds; ++k) {
+    const bool on = k < cnt;
+    const int e = on ? e0 + k : e0;
+    const double x = sddmm_entry<T>(Um, Vm, ld, P.con_r[e], P.con_c[e], P.con_a[e], t);
+    if (on) s += x;
   }
-#pragma unroll
-  for (int kk = 0; kk < KMAX; ++kk)
-#pragma unroll
-    for (int ee = 0; ee < CHUNK; ++ee) out.v[kk][ee] = fma(rho, acc.v[kk][ee], gamma * Pj.v[kk][ee]);
+  return s;
 }
 
 // ------------------------------------------------------------------------------------
@@ -661,24 +772,9 @@ __device__ __forceinline__ void frag_warp_combine(Frag<T>& f, int G) {
     }
 }
 
-// contribution of one A entry (j,k,a) to (H P)_j: a q W_k, q = a (P_j.W_k + P_k.W_j)
-template <typename T>
-__device__ __forceinline__ void hess_entry(const T* Wm, const T* Pm, int ld, int j, int k, T a,
-                                           const Frag<T>& Pj, const Frag<T>& Wj, const Team& t,
-                                           Frag<T>& acc) {
-  if (k == j) {
-    const T q = a * frag_dot(Pj, Wj, t);
-    frag_axpy(acc, a * q, Wj);
-  } else {
-    Frag<T> Wk, Pk;
-    frag_load(Wk, Wm, k, ld, t);
-    frag_load(Pk, Pm, k, ld, t);
-    const T q = a * team_sum(frag_dot_local(Pj, Wk) + frag_dot_local(Pk, Wj), t);
-    frag_axpy(acc, a * q, Wk);
-  }
-}
-
-// (H P)_j = rho sum a q W_k + gamma P_j with the whole warp; out valid in every lane
+// (H P)_j = rho sum a q W_k + gamma P_j with the whole warp; out valid in every lane.  All
+// sub-teams take the same number of rounds, two entries each; an entry past the end of the row has
+// a = 0 and reads nothing.  A diagonal entry (k = j) takes P_k = 0: q = a P_j . W_j.
 template <typename T>
 __device__ void hessian_row_warp(const DevProblem& P, const T* Wm, const T* Pm, int ld, int j,
                                  const Frag<T>& Pj, T rho, T gamma, const WarpRow& w,
@@ -688,27 +784,32 @@ __device__ void hessian_row_warp(const DevProblem& P, const T* Wm, const T* Pm, 
   frag_load(Wj, Wm, j, ld, t);
   frag_zero(acc);
   const T* av = aval<T>(P);
-  const int e0 = P.A_rp[j], e1 = P.A_rp[j + 1];
-  int e = e0 + w.sub;
-  for (; e + w.S < e1; e += 2 * w.S) {
-    const int k0 = P.A_col[e], k1 = P.A_col[e + w.S];
-    const T a0 = av[e], a1 = av[e + w.S];
-    if (k0 != j && k1 != j) {
-      Frag<T> W0, P0, W1, P1;
-      frag_load(W0, Wm, k0, ld, t);
-      frag_load(P0, Pm, k0, ld, t);
-      frag_load(W1, Wm, k1, ld, t);
-      frag_load(P1, Pm, k1, ld, t);
-      const T q0 = a0 * team_sum(frag_dot_local(Pj, W0) + frag_dot_local(P0, Wj), t);
-      const T q1 = a1 * team_sum(frag_dot_local(Pj, W1) + frag_dot_local(P1, Wj), t);
-      frag_axpy(acc, a0 * q0, W0);
-      frag_axpy(acc, a1 * q1, W1);
-    } else {
-      hess_entry(Wm, Pm, ld, j, k0, a0, Pj, Wj, t, acc);
-      hess_entry(Wm, Pm, ld, j, k1, a1, Pj, Wj, t, acc);
+  const int e1 = P.A_rp[j + 1];
+  for (int e0 = P.A_rp[j]; e0 < e1; e0 += 2 * w.S) {
+    Frag<T> Wk[2], Pk[2];
+    T a[2], q[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = e0 + w.sub + h * w.S;
+      Team tw = t, tp = t;
+      int k = j;
+      a[h] = T(0);
+      if (e < e1) {
+        k = P.A_col[e];
+        a[h] = av[e];
+      } else {
+        tw.nc = 0;
+      }
+      tp.nc = k == j ? 0 : tw.nc;
+      frag_load(Wk[h], Wm, k, ld, tw);
+      frag_load(Pk[h], Pm, k, ld, tp);
     }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      q[h] = a[h] * team_sum(frag_dot_local(Pj, Wk[h]) + frag_dot_local(Pk[h], Wj), t);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) frag_axpy(acc, a[h] * q[h], Wk[h]);
   }
-  if (e < e1) hess_entry(Wm, Pm, ld, j, P.A_col[e], av[e], Pj, Wj, t, acc);
   frag_warp_combine(acc, t.G);
 #pragma unroll
   for (int kk = 0; kk < KMAX; ++kk)

@@ -14,7 +14,7 @@ constexpr int SOLVER_THREADS_MIN = 128;   // every solver CTA: four warps, one p
 template <typename T, int SUB>
 __global__ void __launch_bounds__(BLOCK_THREADS_MAX, 1)
 solve_block_kernel(const SolverArgs<T>* args, int count, int* queue) {
-  __shared__ double red[34 * MAXRED];
+  __shared__ double red[RED_ROWS * MAXRED];
   __shared__ SolverArgs<T> sa;
   __shared__ int inst;
   for (;;) {
@@ -33,32 +33,36 @@ solve_block_kernel(const SolverArgs<T>* args, int count, int* queue) {
 // one problem over the whole grid (cooperative launch: all CTAs co-resident)
 template <typename T, int SUB>
 __global__ void __launch_bounds__(GRID_THREADS_MAX, 1)
-solve_grid_kernel(const SolverArgs<T>* args, GridCtl* ctl, double* partials, long long spin) {
-  __shared__ double red[34 * MAXRED];
+solve_grid_kernel(const SolverArgs<T>* args, GridCtl* ctl, Slot* slots, int reps,
+                  long long spin) {
+  __shared__ double red[RED_ROWS * MAXRED];
   __shared__ SolverArgs<T> sa;
   if (threadIdx.x == 0) sa = *args;
-  __syncthreads();
-  GridScope sc{red, ctl, partials, spin, 0, (int)gridDim.x};
+  GridScope sc{red, ctl, slots, reps, spin, 0, (int)gridDim.x};
+  sc.init();
   run_solver<T, SUB>(sa, sc);
 }
 
 // batches with several CTAs per problem: CTAs [g * group, (g + 1) * group) form group g,
 // which takes problems from the queue (largest first) and solves each with a scope spanning
-// the group (ctls[g] is its barrier, slots[g] the index its leader fetched).  The launch is
+// the group (ctls[g] and its share of the slots are its barrier, picks[g] the index its leader
+// fetched).  The launch is
 // cooperative, so every CTA of a group is resident and the group's bounded barriers never
 // wait on a CTA that has not started.
 template <typename T, int SUB>
 __global__ void __launch_bounds__(BLOCK_THREADS_MAX, 1)
 solve_group_kernel(const SolverArgs<T>* args, int count, int* queue, GridCtl* ctls,
-                   double* partials, int* slots, int group, long long spin) {
-  __shared__ double red[34 * MAXRED];
+                   Slot* slots, int* picks, int group, long long spin) {
+  __shared__ double red[RED_ROWS * MAXRED];
   __shared__ SolverArgs<T> sa;
   const int g = blockIdx.x / group;
-  GroupScope sc{{red, ctls + g, partials, spin, g * group, group}};
+  Slot* mine = slots + (size_t)g * group * (SLOT_DOUBLES / 2);
+  GroupScope sc{{red, ctls + g, mine, 1, spin, g * group, group}};
+  sc.init();
   for (;;) {
-    if (sc.is_leader()) slots[g] = atomicAdd(queue, 1);
+    if (sc.is_leader()) picks[g] = atomicAdd(queue, 1);
     if (!sc.sync()) return;
-    const int i = __ldcg(slots + g);
+    const int i = __ldcg(picks + g);
     if (i >= count) return;
     if (threadIdx.x == 0) sa = args[i];
     __syncthreads();
@@ -71,9 +75,9 @@ solve_group_kernel(const SolverArgs<T>* args, int count, int* queue, GridCtl* ct
 template <typename T>
 __global__ void op_sddmm_kernel(DevProblem P, int ld, const T* U, const T* V, double* q) {
   const Team t = make_team(ld, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-  for (int i = t.id; i < P.m; i += t.count) {
-    const double v = sddmm_con<T>(P, U, V, ld, i, t);
-    if (t.lane == 0) q[i] = v;
+  for (TeamRows rows(t, P.m); rows.more(); rows.next()) {
+    const double v = sddmm_con<T>(P, U, V, ld, rows.j, rows.t);
+    if (rows.t.lead) q[rows.j] = v;
   }
 }
 
@@ -104,11 +108,13 @@ __global__ void op_hessian_kernel(DevProblem P, int ld, T rho, T gamma, const T*
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
   if (P.a_diag_only) {
     const Team t = make_team(ld, tid, nt);
-    for (int j = t.id; j < P.n; j += t.count) {
-      Frag<T> Pj, H;
-      frag_load(Pj, Pm, j, ld, t);
-      hessian_row<T>(P, V, Pm, ld, j, Pj, rho, gamma, t, H);
-      frag_store(H, out, j, ld, t);
+    const T* ra = rowa<T>(P);
+    for (TeamRows rows(t, P.n); rows.more(); rows.next()) {
+      Frag<T> Pj, Vj, H;
+      frag_load(Pj, Pm, rows.j, ld, rows.t);
+      frag_load(Vj, V, rows.j, ld, rows.t);
+      hessian_row<T>(ra[rows.j], Vj, Pj, rho, gamma, rows.t, H);
+      frag_store(H, out, rows.j, ld, rows.t);
     }
   } else {
     const WarpRow wr = make_warp_row(ld, tid, nt);
@@ -143,11 +149,11 @@ struct SolveLaunch {
   static cudaError_t solve_block(const SolverArgs<T>* args, int count, int* queue, int grid,
                                  int threads, cudaStream_t s);
   static cudaError_t block_capacity(int threads, int* blocks_per_sm);
-  static cudaError_t solve_grid(const SolverArgs<T>* args, GridCtl* ctl, double* partials,
+  static cudaError_t solve_grid(const SolverArgs<T>* args, GridCtl* ctl, Slot* slots, int reps,
                                 long long spin, int grid, int threads, cudaStream_t s);
   static cudaError_t grid_capacity(int threads, int* blocks_per_sm);
   static cudaError_t solve_group(const SolverArgs<T>* args, int count, int* queue, GridCtl* ctls,
-                                 double* partials, int* slots, int group, long long spin,
+                                 Slot* slots, int* picks, int group, long long spin,
                                  int grid, int threads, cudaStream_t s);
   static cudaError_t group_capacity(int threads, int* blocks_per_sm);
 };
@@ -157,11 +163,11 @@ struct SolveLaunch {
                                                            int, int, cudaStream_t);            \
   template <> cudaError_t SolveLaunch<T, SUB>::block_capacity(int, int*);                      \
   template <> cudaError_t SolveLaunch<T, SUB>::solve_grid(const SolverArgs<T>*, GridCtl*,      \
-                                                          double*, long long, int, int,        \
+                                                          Slot*, int, long long, int, int,     \
                                                           cudaStream_t);                       \
   template <> cudaError_t SolveLaunch<T, SUB>::grid_capacity(int, int*);                       \
   template <> cudaError_t SolveLaunch<T, SUB>::solve_group(const SolverArgs<T>*, int, int*,    \
-                                                           GridCtl*, double*, int*, int,       \
+                                                           GridCtl*, Slot*, int*, int,         \
                                                            long long, int, int, cudaStream_t); \
   template <> cudaError_t SolveLaunch<T, SUB>::group_capacity(int, int*);
 LORADS_DECLARE_SOLVE_LAUNCH(double, 0)
@@ -187,9 +193,9 @@ LORADS_DECLARE_SOLVE_LAUNCH(float, 1)
 #define LORADS_DEFINE_SOLVE_LAUNCH_MULTI(T, SUB)                                               \
   template <>                                                                                  \
   cudaError_t SolveLaunch<T, SUB>::solve_grid(const SolverArgs<T>* args, GridCtl* ctl,         \
-                                              double* partials, long long spin, int grid,      \
+                                              Slot* slots, int reps, long long spin, int grid, \
                                               int threads, cudaStream_t s) {                   \
-    void* kargs[] = {(void*)&args, (void*)&ctl, (void*)&partials, (void*)&spin};               \
+    void* kargs[] = {(void*)&args, (void*)&ctl, (void*)&slots, (void*)&reps, (void*)&spin};    \
     return cudaLaunchCooperativeKernel((const void*)solve_grid_kernel<T, SUB>, dim3(grid),     \
                                        dim3(threads), kargs, 0, s);                            \
   }                                                                                            \
@@ -201,11 +207,11 @@ LORADS_DECLARE_SOLVE_LAUNCH(float, 1)
   }                                                                                            \
   template <>                                                                                  \
   cudaError_t SolveLaunch<T, SUB>::solve_group(const SolverArgs<T>* args, int count,           \
-                                               int* queue, GridCtl* ctls, double* partials,    \
-                                               int* slots, int group, long long spin,          \
+                                               int* queue, GridCtl* ctls, Slot* slots,         \
+                                               int* picks, int group, long long spin,          \
                                                int grid, int threads, cudaStream_t s) {        \
     void* kargs[] = {(void*)&args,     (void*)&count, (void*)&queue, (void*)&ctls,             \
-                     (void*)&partials, (void*)&slots, (void*)&group, (void*)&spin};            \
+                     (void*)&slots,    (void*)&picks, (void*)&group, (void*)&spin};            \
     return cudaLaunchCooperativeKernel((const void*)solve_group_kernel<T, SUB>, dim3(grid),    \
                                        dim3(threads), kargs, 0, s);                            \
   }                                                                                            \
@@ -232,22 +238,22 @@ struct Launch {
     return sub ? SolveLaunch<T, 1>::block_capacity(threads, blocks_per_sm)
                : SolveLaunch<T, 0>::block_capacity(threads, blocks_per_sm);
   }
-  static cudaError_t solve_grid(int sub, const SolverArgs<T>* args, GridCtl* ctl,
-                                double* partials, long long spin, int grid, int threads,
+  static cudaError_t solve_grid(int sub, const SolverArgs<T>* args, GridCtl* ctl, Slot* slots,
+                                int reps, long long spin, int grid, int threads,
                                 cudaStream_t s) {
-    return sub ? SolveLaunch<T, 1>::solve_grid(args, ctl, partials, spin, grid, threads, s)
-               : SolveLaunch<T, 0>::solve_grid(args, ctl, partials, spin, grid, threads, s);
+    return sub ? SolveLaunch<T, 1>::solve_grid(args, ctl, slots, reps, spin, grid, threads, s)
+               : SolveLaunch<T, 0>::solve_grid(args, ctl, slots, reps, spin, grid, threads, s);
   }
   static cudaError_t grid_capacity(int sub, int threads, int* blocks_per_sm) {
     return sub ? SolveLaunch<T, 1>::grid_capacity(threads, blocks_per_sm)
                : SolveLaunch<T, 0>::grid_capacity(threads, blocks_per_sm);
   }
   static cudaError_t solve_group(int sub, const SolverArgs<T>* args, int count, int* queue,
-                                 GridCtl* ctls, double* partials, int* slots, int group,
+                                 GridCtl* ctls, Slot* slots, int* picks, int group,
                                  long long spin, int grid, int threads, cudaStream_t s) {
-    return sub ? SolveLaunch<T, 1>::solve_group(args, count, queue, ctls, partials, slots,
+    return sub ? SolveLaunch<T, 1>::solve_group(args, count, queue, ctls, slots, picks,
                                                 group, spin, grid, threads, s)
-               : SolveLaunch<T, 0>::solve_group(args, count, queue, ctls, partials, slots,
+               : SolveLaunch<T, 0>::solve_group(args, count, queue, ctls, slots, picks,
                                                 group, spin, grid, threads, s);
   }
   static cudaError_t group_capacity(int sub, int threads, int* blocks_per_sm) {

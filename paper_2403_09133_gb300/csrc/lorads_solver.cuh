@@ -228,7 +228,8 @@ struct Solver {
   __device__ T* dir_shadow() const {
     return ((const void*)A.Ut == (const void*)A.U) ? reinterpret_cast<T*>(A.dir) : A.Dl;
   }
-  __device__ __forceinline__ void store_shadow(const Frag<double>& f, T* dst, int j) const {
+  __device__ __forceinline__ void store_shadow(const Frag<double>& f, T* dst, int j,
+                                               const Team& tm) const {
     if ((const void*)dst == (const void*)A.U || (const void*)dst == (const void*)A.dir) return;
     Frag<T> t;
     frag_convert(t, f);
@@ -238,7 +239,9 @@ struct Solver {
   __device__ void init_factor() {
     const uint64_t key = stream_key(prm.seed, 0);
     const double inv = 1.0 / sqrt((double)r);
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> f;
 #pragma unroll
       for (int k = 0; k < KMAX; ++k)
@@ -247,8 +250,9 @@ struct Solver {
           const int c = (tm.lane + k * tm.G) * CHUNK + e;
           f.v[k][e] = (c < r) ? normal_at(key, (uint64_t)j * r + c) * inv : 0.0;
         }
+      const double f2 = P.row_norm != nullptr ? frag_dot(f, f, tm) : 0.0;
       if (P.row_norm != nullptr && P.row_norm[j] > 0.0) {
-        const double nr = sqrt(frag_dot(f, f, tm));
+        const double nr = sqrt(f2);
         const double s = P.row_norm[j] / nr;
 #pragma unroll
         for (int k = 0; k < KMAX; ++k)
@@ -256,26 +260,37 @@ struct Solver {
           for (int e = 0; e < CHUNK; ++e) f.v[k][e] *= s;
       }
       frag_store(f, A.U, j, ld, tm);
-      store_shadow(f, A.Ut, j);
+      store_shadow(f, A.Ut, j, tm);
     }
   }
 
   // ----------------------------------------------------------------------------------
   // Multi-entry constraints: the products <A_i, X Y^T> are sums over each constraint's
   // entries.  One team per chunk of at most CON_CHUNK entries forms K per-entry sums
-  // f(r, c, a, s) at once (so a long constraint such as tr X = 1 is spread over many teams);
+  // f(r, c, a, team, s) at once (so a long constraint such as tr X = 1 is spread over many teams);
   // after a barrier, con_total(i, k) adds constraint i's chunks in a fixed order.
   // ----------------------------------------------------------------------------------
   template <int K, typename F>
   __device__ bool con_chunks(F f) {
     const int nch = P.nchunk;
-    for (int ch = tmc.id; ch < nch; ch += tmc.count) {
+    for (TeamRows rows(this->tmc, nch); rows.more(); rows.next()) {
+      const Team& tmc = rows.t;
+      const int ch = rows.j, e0 = P.chunk_ptr[ch];
+      const int cnt = tmc.live ? P.chunk_ptr[ch + 1] - e0 : 0;
+      const int rounds = __reduce_max_sync(0xffffffffu, cnt);   // the warp's teams stay together
       double s[K];
 #pragma unroll
       for (int k = 0; k < K; ++k) s[k] = 0.0;
-      for (int e = P.chunk_ptr[ch]; e < P.chunk_ptr[ch + 1]; ++e)
-        f(P.con_r[e], P.con_c[e], P.con_a[e], s);
-      if (tmc.lane == 0) {
+      for (int t = 0; t < rounds; ++t) {
+        const bool on = t < cnt;
+        const int e = on ? e0 + t : e0;
+        double x[K];
+        f(P.con_r[e], P.con_c[e], P.con_a[e], tmc, x);
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+          if (on) s[k] += x[k];
+      }
+      if (tmc.lead) {
 #pragma unroll
         for (int k = 0; k < K; ++k) A.cq[(long long)k * nch + ch] = s[k];
       }
@@ -293,8 +308,8 @@ struct Solver {
   // q_i = <A_i, X Y^T> for every constraint into A.cq + 3 nchunk, visible to the whole scope
   template <typename E>
   __device__ bool con_q(const E* X, const E* Y) {
-    if (!con_chunks<1>([&](int r, int c, double a, double* s) {
-          s[0] += sddmm_entry<E>(X, Y, ld, r, c, a, tmc);
+    if (!con_chunks<1>([&](int r, int c, double a, const Team& tmc, double* s) {
+          s[0] = sddmm_entry<E>(X, Y, ld, r, c, a, tmc);
         }))
       return false;
     double* q = A.cq + 3LL * P.nchunk;
@@ -320,8 +335,8 @@ struct Solver {
   __device__ bool eval_residual_UU_e(const E* Ub, double& e2) {
     double v[1] = {0.0};
     if (P.a_multi) {
-      if (!con_chunks<1>([&](int r, int c, double a, double* s) {
-            s[0] += sddmm_entry<E>(Ub, Ub, ld, r, c, a, tmc);
+      if (!con_chunks<1>([&](int r, int c, double a, const Team& tmc, double* s) {
+            s[0] = sddmm_entry<E>(Ub, Ub, ld, r, c, a, tmc);
           }))
         return false;
       for (int i = sc.tid(); i < m; i += sc.nthreads()) {
@@ -330,10 +345,12 @@ struct Solver {
         v[0] += ei * ei;
       }
     } else {
-      for (int i = tmc.id; i < m; i += tmc.count) {
+      for (TeamRows rows(this->tmc, m); rows.more(); rows.next()) {
+        const Team& tmc = rows.t;
+        const int i = rows.j;
         const double q = sddmm_con<E>(P, Ub, Ub, ld, i, tmc);
         const double ei = q - P.b[i];
-        if (tmc.lane == 0) {
+        if (tmc.lead) {
           A.e[i] = ei;
           v[0] += ei * ei;
         }
@@ -353,7 +370,9 @@ struct Solver {
   __device__ bool eval_grad_e(const E* Ub, double sigma, double& g2) {
     double v[1] = {0.0};
     if (P.a_diag_only) {
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<E> ot;
         Frag<double> out;
         spmm_row<E>(P, Ub, ld, j, A.lam, A.e, 0.0, -1.0, -sigma, E(0), tm, ot);
@@ -364,7 +383,7 @@ struct Solver {
           for (int e = 0; e < CHUNK; ++e) out.v[k][e] *= -2.0;
         frag_store(out, A.grad, j, ld, tm);
         const double d = frag_dot(out, out, tm);
-        if (tm.lane == 0) v[0] += d;
+        if (tm.lead) v[0] += d;
       }
     } else {
       // rows with many entries: one warp per row
@@ -374,15 +393,13 @@ struct Solver {
         Frag<double> out;
         spmm_row_warp<E>(P, Ub, ld, j, A.lam, A.e, 0.0, -1.0, -sigma, E(0), wr, ot);
         frag_convert(out, ot);
-        if (wr.sub == 0) {
 #pragma unroll
-          for (int k = 0; k < KMAX; ++k)
+        for (int k = 0; k < KMAX; ++k)
 #pragma unroll
-            for (int e = 0; e < CHUNK; ++e) out.v[k][e] *= -2.0;
-          frag_store(out, A.grad, j, ld, wr.st);
-          const double d = frag_dot(out, out, wr.st);
-          if (wr.st.lane == 0) v[0] += d;
-        }
+          for (int e = 0; e < CHUNK; ++e) out.v[k][e] *= -2.0;
+        if (wr.sub == 0) frag_store(out, A.grad, j, ld, wr.st);
+        const double d = frag_dot(out, out, wr.st);
+        if (wr.sub == 0 && wr.st.lead) v[0] += d;
       }
     }
     if (!sc.reduce(v, 1)) return false;
@@ -405,7 +422,9 @@ struct Solver {
     double alpha[MAXMEM + 1], beta_prev = 0.0;
     if (cnt == 0) {
       double v[1] = {0.0};
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<double> g;
         frag_load(g, A.grad, j, ld, tm);
 #pragma unroll
@@ -413,9 +432,9 @@ struct Solver {
 #pragma unroll
           for (int e = 0; e < CHUNK; ++e) g.v[k][e] = -g.v[k][e];
         frag_store(g, A.dir, j, ld, tm);
-        store_shadow(g, dir_shadow(), j);
+        store_shadow(g, dir_shadow(), j, tm);
         const double d = frag_dot(g, g, tm);
-        if (tm.lane == 0) v[0] -= d;
+        if (tm.lead) v[0] -= d;
       }
       if (!sc.reduce(v, 1)) return false;
       dg = v[0];
@@ -426,7 +445,9 @@ struct Solver {
       const int slot = (head - 1 - i + 2 * mem) % mem;
       const int prev = (head - i + 2 * mem) % mem;   // slot of pair i-1
       double v[1] = {0.0};
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<double> q, s;
         if (i == 0) {
           frag_load(q, A.grad, j, ld, tm);
@@ -439,7 +460,7 @@ struct Solver {
         frag_store(q, A.dir, j, ld, tm);
         frag_load(s, A.S + slot * NS, j, ld, tm);
         const double d = frag_dot(s, q, tm);
-        if (tm.lane == 0) v[0] += d;
+        if (tm.lead) v[0] += d;
       }
       if (!sc.reduce(v, 1)) return false;
       alpha[i] = hrho[slot] * v[0];
@@ -449,7 +470,9 @@ struct Solver {
       const int slot = (head - cnt + i + 2 * mem) % mem;
       const int ai = cnt - 1 - i;
       double v[1] = {0.0};
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<double> q;
         frag_load(q, A.dir, j, ld, tm);
         if (i == 0) {
@@ -470,7 +493,7 @@ struct Solver {
         Frag<double> y;
         frag_load(y, A.Y + slot * NS, j, ld, tm);
         const double d = frag_dot(y, q, tm);
-        if (tm.lane == 0) v[0] += d;
+        if (tm.lead) v[0] += d;
       }
       if (!sc.reduce(v, 1)) return false;
       beta_prev = hrho[slot] * v[0];
@@ -478,7 +501,9 @@ struct Solver {
     {
       const int last = (head - 1 + 2 * mem) % mem;
       double v[1] = {0.0};
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<double> q, s, g;
         frag_load(q, A.dir, j, ld, tm);
         frag_load(s, A.S + last * NS, j, ld, tm);
@@ -488,10 +513,10 @@ struct Solver {
 #pragma unroll
           for (int e = 0; e < CHUNK; ++e) q.v[k][e] = -q.v[k][e];
         frag_store(q, A.dir, j, ld, tm);
-        store_shadow(q, dir_shadow(), j);
+        store_shadow(q, dir_shadow(), j, tm);
         frag_load(g, A.grad, j, ld, tm);
         const double d = frag_dot(q, g, tm);
-        if (tm.lane == 0) v[0] += d;
+        if (tm.lead) v[0] += d;
       }
       if (!sc.reduce(v, 1)) return false;
       dg = v[0];
@@ -501,7 +526,9 @@ struct Solver {
 
   // dir <- -grad (restart)
   __device__ bool steepest() {
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> g;
       frag_load(g, A.grad, j, ld, tm);
 #pragma unroll
@@ -509,7 +536,7 @@ struct Solver {
 #pragma unroll
         for (int e = 0; e < CHUNK; ++e) g.v[k][e] = -g.v[k][e];
       frag_store(g, A.dir, j, ld, tm);
-      store_shadow(g, dir_shadow(), j);
+      store_shadow(g, dir_shadow(), j, tm);
     }
     return sc.sync();
   }
@@ -521,14 +548,16 @@ struct Solver {
 #pragma unroll
     for (int i = 0; i < 9; ++i) v[i] = 0.0;
     // <C, U D^T + D U^T> = 2 sum_j D_j . (C U)_j ;  <C, D D^T> = sum_j D_j . (C D)_j
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<E> mCU, mCD, Dj;
       spmm_row<E>(P, Ub, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, E(0), tm, mCU);
       spmm_row<E>(P, Dt, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, E(0), tm, mCD);
       frag_load(Dj, Dt, j, ld, tm);
       const double c1 = -2.0 * (double)frag_dot(Dj, mCU, tm);
       const double c2 = -(double)frag_dot(Dj, mCD, tm);
-      if (tm.lane == 0) {
+      if (tm.lead) {
         v[7] += c1;
         v[8] += c2;
       }
@@ -545,14 +574,16 @@ struct Solver {
       v[6] += e2 * e2;
     };
     if (P.a_multi) {
-      if (!con_chunks<2>([&](int r, int c, double a, double* s) {
-            s[0] += 2.0 * sddmm_entry<E>(Ub, Dt, ld, r, c, a, tmc);
-            s[1] += sddmm_entry<E>(Dt, Dt, ld, r, c, a, tmc);
+      if (!con_chunks<2>([&](int r, int c, double a, const Team& tmc, double* s) {
+            s[0] = 2.0 * sddmm_entry<E>(Ub, Dt, ld, r, c, a, tmc);
+            s[1] = sddmm_entry<E>(Dt, Dt, ld, r, c, a, tmc);
           }))
         return false;
       for (int i = sc.tid(); i < m; i += sc.nthreads()) accumulate(i, con_total(i, 0), con_total(i, 1));
     } else {
-      for (int i = tmc.id; i < m; i += tmc.count) {
+      for (TeamRows rows(this->tmc, m); rows.more(); rows.next()) {
+        const Team& tmc = rows.t;
+        const int i = rows.j;
         const int rr = P.con_r[i], cc = P.con_c[i];
         const double aa = P.con_a[i];
         Frag<E> Ur, Dc, Dr, Uc;
@@ -560,15 +591,11 @@ struct Solver {
         frag_load(Dc, Dt, cc, ld, tmc);
         frag_load(Dr, Dt, rr, ld, tmc);
         frag_load(Uc, Ub, cc, ld, tmc);
-        double e1, e2;
-        if (rr != cc) {
-          e1 = 2.0 * aa * (double)team_sum(frag_dot_local(Ur, Dc) + frag_dot_local(Uc, Dr), tmc);
-          e2 = 2.0 * aa * (double)frag_dot(Dr, Dc, tmc);
-        } else {
-          e1 = 2.0 * aa * (double)frag_dot(Ur, Dr, tmc);
-          e2 = aa * (double)frag_dot(Dr, Dr, tmc);
-        }
-        if (tmc.lane == 0) accumulate(i, e1, e2);
+        E loc = frag_dot_local(Ur, Dc);
+        if (rr != cc) loc += frag_dot_local(Uc, Dr);
+        const double e1 = 2.0 * aa * (double)team_sum(loc, tmc);
+        const double e2 = (rr != cc ? 2.0 : 1.0) * aa * (double)frag_dot(Dr, Dc, tmc);
+        if (tmc.lead) accumulate(i, e1, e2);
       }
     }
     if (!sc.reduce(v, 9)) return false;
@@ -587,7 +614,9 @@ struct Solver {
   // U <- U + t dir; S[head] = t dir; grad_old = grad
   __device__ bool take_step(double t, int head) {
     const long long NS = (long long)n * A.ld_cap;
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> u, d, g;
       frag_load(u, A.U, j, ld, tm);
       frag_load(d, A.dir, j, ld, tm);
@@ -597,7 +626,7 @@ struct Solver {
         for (int e = 0; e < CHUNK; ++e) d.v[k][e] *= t;
       frag_axpy(u, 1.0, d);
       frag_store(u, A.U, j, ld, tm);
-      store_shadow(u, A.Ut, j);
+      store_shadow(u, A.Ut, j, tm);
       frag_store(d, A.S + head * NS, j, ld, tm);
       frag_load(g, A.grad, j, ld, tm);
       frag_store(g, A.grad_old, j, ld, tm);
@@ -609,7 +638,9 @@ struct Solver {
   __device__ bool history_pair(int head, double& sy, double& yy) {
     const long long NS = (long long)n * A.ld_cap;
     double v[2] = {0.0, 0.0};
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> g, go, s;
       frag_load(g, A.grad, j, ld, tm);
       frag_load(go, A.grad_old, j, ld, tm);
@@ -617,7 +648,7 @@ struct Solver {
       frag_store(g, A.Y + head * NS, j, ld, tm);
       frag_load(s, A.S + head * NS, j, ld, tm);
       const double a = frag_dot(s, g, tm), b = frag_dot(g, g, tm);
-      if (tm.lane == 0) {
+      if (tm.lead) {
         v[0] += a;
         v[1] += b;
       }
@@ -641,7 +672,9 @@ struct Solver {
     set_rank(r_new);
     const uint64_t key = stream_key(prm.seed, (uint64_t)g);
     const int extra = r_new - r_old;
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> u;
 #pragma unroll
       for (int k = 0; k < KMAX; ++k)
@@ -656,7 +689,7 @@ struct Solver {
           u.v[k][e] = x;
         }
       frag_store(u, A.U, j, ld, tm);
-      store_shadow(u, A.Ut, j);
+      store_shadow(u, A.Ut, j, tm);
     }
     return sc.sync();
   }
@@ -779,9 +812,13 @@ struct Solver {
       frag_load(Wj, Wm, j, ld, st);
       frag_zero(accR);
       frag_zero(accG);
-      for (int q = P.A_rp[j] + wr.sub; q < P.A_rp[j + 1]; q += wr.S) {
-        const int k = P.A_col[q], i = P.A_con[q];
-        const double a = P.A_val[q];
+      // every sub-team takes the same number of rounds (team sums name the whole warp)
+      const int q1 = P.A_rp[j + 1];
+      for (int q0 = P.A_rp[j]; q0 < q1; q0 += wr.S) {
+        const int q = q0 + wr.sub;
+        const bool on = q < q1;
+        const int k = on ? P.A_col[q] : j, i = on ? P.A_con[q] : 0;
+        const double a = on ? P.A_val[q] : 0.0;
         double qi;
         Frag<double> Wk;
         if (k == j)
@@ -792,9 +829,11 @@ struct Solver {
           qi = qv[i];
         else
           qi = (k == j ? 1.0 : 2.0) * a * frag_dot(Wj, Wk, st);
-        const double w = rho * P.b[i] - A.lam[i];
-        frag_axpy(accG, a * w, Wk);
-        frag_axpy(accR, a * (w - rho * qi), Wk);
+        if (on) {
+          const double w = rho * P.b[i] - A.lam[i];
+          frag_axpy(accG, a * w, Wk);
+          frag_axpy(accR, a * (w - rho * qi), Wk);
+        }
       }
       for (int q = P.C_rp[j] + wr.sub; q < P.C_rp[j + 1]; q += wr.S) {
         Frag<double> Wk;
@@ -805,20 +844,20 @@ struct Solver {
       frag_warp_combine(accR, st.G);
       frag_warp_combine(accG, st.G);
       frag_axpy(accG, gamma, Wj);
+      Frag<T> Rt, Zt;
+      frag_convert(Rt, accR);
+      frag_zero(Zt);
       if (wr.sub == 0) {
-        Frag<T> Rt, Zt;
-        frag_convert(Rt, accR);
-        frag_zero(Zt);
         frag_store(Rt, A.R, j, ld, st);
         frag_store(Rt, A.Pd, j, ld, st);
         frag_store(Zt, A.Dl, j, ld, st);
-        Frag<double> Rd;
-        frag_convert(Rd, Rt);
-        const double a1 = frag_dot(Rd, Rd, st), a2 = frag_dot(accG, accG, st);
-        if (st.lane == 0) {
-          v[0] += a1;
-          v[1] += a2;
-        }
+      }
+      Frag<double> Rd;
+      frag_convert(Rd, Rt);
+      const double a1 = frag_dot(Rd, Rd, st), a2 = frag_dot(accG, accG, st);
+      if (wr.sub == 0 && st.lead) {
+        v[0] += a1;
+        v[1] += a2;
       }
     }
     if (!sc.reduce(v, 2)) return false;
@@ -838,11 +877,9 @@ struct Solver {
           hessian_row_q_warp<T>(P, Wt, ld, j, Pj, qv, rho_t, gamma_t, wr, Hj);
         else
           hessian_row_warp<T>(P, Wt, A.Pd, ld, j, Pj, rho_t, gamma_t, wr, Hj);
-        if (wr.sub == 0) {
-          frag_store(Hj, A.HP, j, ld, st);
-          const double d = (double)team_sum(frag_dot_local(Pj, Hj), st);
-          if (st.lane == 0) w[0] += d;
-        }
+        if (wr.sub == 0) frag_store(Hj, A.HP, j, ld, st);
+        const T d = team_sum(frag_dot_local(Pj, Hj), st);
+        if (wr.sub == 0 && st.lead) w[0] += (double)d;
       }
       if (!sc.reduce(w, 1)) return false;
       ++hess;
@@ -854,7 +891,9 @@ struct Solver {
       const double alpha = rr / pHp;
       const T alpha_t = (T)alpha;
       double z[1] = {0.0};
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<T> Dj, Pj, Rj, Hj;
         frag_load(Dj, A.Dl, j, ld, tm);
         frag_load(Pj, A.Pd, j, ld, tm);
@@ -867,7 +906,7 @@ struct Solver {
         Frag<double> Rd;
         frag_convert(Rd, Rj);
         const double d = frag_dot(Rd, Rd, tm);
-        if (tm.lane == 0) z[0] += d;
+        if (tm.lead) z[0] += d;
       }
       if (!sc.reduce(z, 1)) return false;
       ++it;
@@ -875,7 +914,9 @@ struct Solver {
       if (sqrt(rr_new) <= target) { rr = rr_new; break; }
       const T beta_t = (T)(rr_new / rr);
       rr = rr_new;
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<T> Pj, Rj;
         frag_load(Pj, A.Pd, j, ld, tm);
         frag_load(Rj, A.R, j, ld, tm);
@@ -891,7 +932,9 @@ struct Solver {
     // X = W + delta (FP64 master and T shadow)
     dv[0] = 0.0;
     dv[1] = 0.0;
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> Wj, Xj;
       Frag<T> Dj;
       frag_load(Wj, Wm, j, ld, tm);
@@ -904,7 +947,7 @@ struct Solver {
         const double o2 = frag_dot(Xo, Xo, tm);
         frag_axpy(Xo, -1.0, Xj);
         const double d2 = frag_dot(Xo, Xo, tm);
-        if (tm.lane == 0) {
+        if (tm.lead) {
           dv[0] += d2;
           dv[1] += o2;
         }
@@ -927,7 +970,7 @@ struct Solver {
   // are independent (phase2_local below).
   // ----------------------------------------------------------------------------------
   __device__ __forceinline__ void local_h(const Frag<T>& x, const Frag<T>& Wj, T a, T rho,
-                                          T gamma, Frag<T>& out) const {
+                                          T gamma, const Team& tm, Frag<T>& out) const {
     const T q = rho * a * a * frag_dot(x, Wj, tm);
 #pragma unroll
     for (int k = 0; k < KMAX; ++k)
@@ -938,7 +981,7 @@ struct Solver {
   // dual step lambda += rho (A(U V^T) - b); partial sums of ||e||^2 and of the output
   // infeasibility ||A(U_hat U_hat^T) - b||^2, U_hat = (U + V)/2
   // entry (r, c, a) of a constraint: its terms of <A_i, U V^T> and <A_i, U_hat U_hat^T>
-  __device__ __forceinline__ void dual_entry(int rr, int cc, double a, double& q,
+  __device__ __forceinline__ void dual_entry(int rr, int cc, double a, const Team& tmc, double& q,
                                              double& qh) const {
     Frag<double> Ur, Vc, Uc, Vr;
     frag_load(Ur, A.U, rr, ld, tmc);
@@ -948,13 +991,11 @@ struct Solver {
     Frag<double> Hr = Ur, Hc = Uc;
     frag_axpy(Hr, 1.0, Vr);
     frag_axpy(Hc, 1.0, Vc);
-    if (rr != cc) {
-      q = a * team_sum(frag_dot_local(Ur, Vc) + frag_dot_local(Uc, Vr), tmc);
-      qh = 0.5 * a * frag_dot(Hr, Hc, tmc);      // 2 (Hr/2).(Hc/2)
-    } else {
-      q = a * frag_dot(Ur, Vr, tmc);
-      qh = 0.25 * a * frag_dot(Hr, Hr, tmc);
-    }
+    double loc = frag_dot_local(Ur, Vc);
+    if (rr != cc) loc += frag_dot_local(Uc, Vr);
+    q = a * team_sum(loc, tmc);
+    // off the diagonal 2 (Hr/2).(Hc/2), on it (Hr/2).(Hr/2)
+    qh = (rr != cc ? 0.5 : 0.25) * a * frag_dot(Hr, Hc, tmc);
   }
 
   __device__ bool dual_step(double rho, double* v) {
@@ -965,20 +1006,19 @@ struct Solver {
       v[1] += eh * eh;
     };
     if (P.a_multi) {
-      if (!con_chunks<2>([&](int r, int c, double a, double* s) {
-            double q, qh;
-            dual_entry(r, c, a, q, qh);
-            s[0] += q;
-            s[1] += qh;
+      if (!con_chunks<2>([&](int r, int c, double a, const Team& tmc, double* s) {
+            dual_entry(r, c, a, tmc, s[0], s[1]);
           }))
         return false;
       for (int i = sc.tid(); i < m; i += sc.nthreads()) update(i, con_total(i, 0), con_total(i, 1));
       return true;
     }
-    for (int i = tmc.id; i < m; i += tmc.count) {
+    for (TeamRows rows(this->tmc, m); rows.more(); rows.next()) {
+      const Team& tmc = rows.t;
+      const int i = rows.j;
       double q, qh;
-      dual_entry(P.con_r[i], P.con_c[i], P.con_a[i], q, qh);
-      if (tmc.lane == 0) update(i, q, qh);
+      dual_entry(P.con_r[i], P.con_c[i], P.con_a[i], tmc, q, qh);
+      if (tmc.lead) update(i, q, qh);
     }
     return true;
   }
@@ -1157,11 +1197,12 @@ struct Solver {
   __device__ __forceinline__ double local_r0_row(int j, const Frag<double>& Wj, const Frag<T>& Wjt,
                                                  const Frag<double>& mCWj, const RowCon& c,
                                                  double lam_i, double rho, double gamma,
-                                                 double* g3, T* dout = nullptr) {
+                                                 const Team& tm, double* g3, T* dout = nullptr) {
     Frag<double> accR = mCWj;
     double cg = gamma, qi = 0.0;
+    const double w2 = frag_dot(Wj, Wj, tm);
     if (c.i >= 0) {
-      qi = c.a * frag_dot(Wj, Wj, tm);
+      qi = c.a * w2;
       frag_axpy(accR, c.a * (rho * c.b - lam_i - rho * qi), Wj);
       cg += c.a * rho * qi;
     }
@@ -1180,14 +1221,14 @@ struct Solver {
       frag_store(wt, dout, j, ld, tm);
       return qi;
     }
-    local_h(rt, Wjt, at, (T)rho, (T)gamma, wt);
+    local_h(rt, Wjt, at, (T)rho, (T)gamma, tm, wt);
     frag_store(rt, A.R, j, ld, tm);
     frag_store(wt, A.HP, j, ld, tm);
     gt = rt;
     frag_axpy(gt, (T)cg, Wjt);
     const double d1 = (double)frag_dot(rt, rt, tm), d2 = (double)frag_dot(wt, rt, tm);
     const double d3 = (double)frag_dot(gt, gt, tm);
-    if (tm.lane == 0) {
+    if (tm.lead) {
       g3[0] += d1;
       g3[1] += d2;
       g3[2] += d3;
@@ -1199,7 +1240,8 @@ struct Solver {
   // neighbours' W and delta when exact, else mCWj - (C delta)_j with the product in T
   __device__ __forceinline__ void local_mcx_row(int j, const double* Wm, const T* D,
                                                 bool have_delta, bool exact,
-                                                const Frag<double>& mCWj, Frag<double>& out) {
+                                                const Frag<double>& mCWj, const Team& tm,
+                                                Frag<double>& out) {
     if (exact) {
       Frag<double> acc;
       frag_zero(acc);
@@ -1233,16 +1275,18 @@ struct Solver {
   __device__ bool local_prologue(double rho, double gamma, double* g3, T* dout = nullptr) {
     g3[0] = g3[1] = g3[2] = 0.0;
     const bool shadow = (const void*)A.Vt != (const void*)A.V;
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       const RowCon c = row_con_of(j);
       Frag<double> Wj, mCW;
       Frag<T> Wjt;
       frag_load(Wj, A.V, j, ld, tm);
       if (shadow) frag_load(Wjt, A.Vt, j, ld, tm);
       else frag_convert(Wjt, Wj);
-      local_mcx_row(j, A.V, A.Dl, false, true, Wj, mCW);
+      local_mcx_row(j, A.V, A.Dl, false, true, Wj, tm, mCW);
       frag_store(mCW, A.CWn, j, ld, tm);
-      local_r0_row(j, Wj, Wjt, mCW, c, c.lam, rho, gamma, g3, dout);
+      local_r0_row(j, Wj, Wjt, mCW, c, c.lam, rho, gamma, tm, g3, dout);
     }
     if (!sc.reduce(g3, 3)) return false;
     ++hess;
@@ -1258,7 +1302,7 @@ struct Solver {
   // row j of the in-memory row-local CG step: its r, p, x (p, x zero on the first step) and W
   __device__ __forceinline__ void cg7_load(int j, bool have_px, Frag<T>& r, Frag<T>& pp,
                                            Frag<T>& x, Frag<T>& Wjt, T& aj, const T* Wt,
-                                           const T* ra) const {
+                                           const T* ra, const Team& tm) const {
     frag_load(r, A.R, j, ld, tm);
     frag_load(Wjt, Wt, j, ld, tm);
     aj = ra[j];
@@ -1270,16 +1314,30 @@ struct Solver {
       frag_zero(x);
     }
   }
+  // two sums over rows, carried by the teams in reduce_pair's form: teams of two or more lanes
+  // keep the first sum in their even lanes' z0 and the second in their odd lanes', one FP64
+  // conversion and addition for both (FP64 runs at 1/64 of FP32 here); single lanes keep both
+  __device__ __forceinline__ void pair_add(T d1, T d2, const Team& tm, double& z0,
+                                           double& z1) const {
+    if (!tm.live) return;
+    if (tm.G >= 2) {
+      z0 += (double)((tm.lane & 1) ? d2 : d1);
+    } else {
+      z0 += (double)d1;
+      z1 += (double)d2;
+    }
+  }
   // p = r + b p, s = H p, x += a p, r -= a s, w = H r; stores p, x, r; z += (r.r, w.r)
   __device__ __forceinline__ void cg7_step(int j, Frag<T>& r, Frag<T>& pp, Frag<T>& x,
                                            const Frag<T>& Wjt, T aj, T a_t, T b_t, T rho_t,
-                                           T gamma_t, double* z) const {
+                                           T gamma_t, const Team& tm, double& z0,
+                                           double& z1) const {
     Frag<T> ss, w;
 #pragma unroll
     for (int k = 0; k < KMAX; ++k)
 #pragma unroll
       for (int e = 0; e < CHUNK; ++e) pp.v[k][e] = fma(b_t, pp.v[k][e], r.v[k][e]);
-    local_h(pp, Wjt, aj, rho_t, gamma_t, ss);
+    local_h(pp, Wjt, aj, rho_t, gamma_t, tm, ss);
 #pragma unroll
     for (int k = 0; k < KMAX; ++k)
 #pragma unroll
@@ -1287,125 +1345,44 @@ struct Solver {
         x.v[k][e] = fma(a_t, pp.v[k][e], x.v[k][e]);
         r.v[k][e] = fma(-a_t, ss.v[k][e], r.v[k][e]);
       }
-    local_h(r, Wjt, aj, rho_t, gamma_t, w);
+    local_h(r, Wjt, aj, rho_t, gamma_t, tm, w);
     frag_store(pp, A.Pd, j, ld, tm);
     frag_store(x, A.Dl, j, ld, tm);
     frag_store(r, A.R, j, ld, tm);
     const T d1 = frag_dot(r, r, tm), d2 = frag_dot(w, r, tm);
-    if (tm.lane == 0) {
-      z[0] += (double)d1;
-      z[1] += (double)d2;
-    }
+    pair_add(d1, d2, tm, z0, z1);
   }
 
   __device__ bool cg_local_loop(const T* Wt, double rho, double gamma, const double* g3,
                                 int& it) {
     const T rho_t = (T)rho, gamma_t = (T)gamma;
     const T* ra = rowa<T>(P);
-    const bool lead = threadIdx.x == 0;
-    double* shs = sc.scratch() + 4;   // state (0 go on, 1 stop, 2 NaN), alpha, beta
     // thread 0 carries gamma = r.r and ga = gamma * alpha: with D = delta_new ga - gamma_new^2
     // the Chronopoulos-Gear update alpha_new = gamma_new / (delta_new - beta gamma_new / alpha)
     // is gamma_new ga / D and beta = gamma_new / gamma = gamma_new D / (gamma D), both from the
     // one reciprocal 1 / (gamma D) (the denominator is positive exactly when D is)
-    double gam = 0.0, ga = 0.0, target2 = 0.0;
-    if (lead) {
+    // (kept in shared memory: a register that only thread 0 uses costs every thread one)
+    double& gam = sc.scratch()[12];
+    double& ga = sc.scratch()[13];
+    double& target2 = sc.scratch()[14];
+    if (threadIdx.x == 0) {
       gam = g3[0];
       const double del = g3[1];
       target2 = fmax(prm.cg_rel_tol * prm.cg_rel_tol * gam,
                      prm.cg_abs_floor * prm.cg_abs_floor * g3[2]);
       const double alpha = del > 0.0 ? gam / del : 0.0;
       ga = gam * alpha;
-      shs[0] = (gam > target2 && del > 0.0) ? 0.0 : 1.0;
-      shs[1] = alpha;
-      shs[2] = 0.0;
+      cg_leave((gam > target2 && del > 0.0) ? 0 : 1, alpha, 0.0);
     }
     __syncthreads();
-    int go = shs[0] == 0.0;
-    T a_t = (T)shs[1], b_t = T(0);
-    __syncthreads();
-    it = 0;
-    if (tm.count >= n) {
-      // at most one row per team: its CG state stays in registers across the iterations
-      // (same arithmetic in the same order as below), and only delta is stored at the end
-      const int j = tm.id;
-      const bool have = j < n;
-      Frag<T> r, w, pp, ss, x, Wjt;
-      T aj = T(0);
-      frag_zero(pp);
-      frag_zero(ss);
-      frag_zero(x);
-      if (have) {
-        frag_load(r, A.R, j, ld, tm);
-        frag_load(w, A.HP, j, ld, tm);
-        frag_load(Wjt, Wt, j, ld, tm);
-        aj = ra[j];
-      } else {
-        frag_zero(r);
-        frag_zero(w);
-        frag_zero(Wjt);
-      }
-      while (go && it < prm.cg_max_iter) {
-        double z[2] = {0.0, 0.0};
-        if (have) {
-#pragma unroll
-          for (int k = 0; k < KMAX; ++k)
-#pragma unroll
-            for (int e = 0; e < CHUNK; ++e) {
-              pp.v[k][e] = fma(b_t, pp.v[k][e], r.v[k][e]);
-              ss.v[k][e] = fma(b_t, ss.v[k][e], w.v[k][e]);
-              x.v[k][e] = fma(a_t, pp.v[k][e], x.v[k][e]);
-              r.v[k][e] = fma(-a_t, ss.v[k][e], r.v[k][e]);
-            }
-          local_h(r, Wjt, aj, rho_t, gamma_t, w);
-          const T d1 = frag_dot(r, r, tm), d2 = frag_dot(w, r, tm);
-          if (tm.lane == 0) {
-            z[0] += (double)d1;
-            z[1] += (double)d2;
-          }
-        }
-        if (!sc.reduce(z, 2)) return false;
-        ++hess;
-        ++it;
-        if (!cg_scalars(lead, shs, z, target2, gam, ga, go, a_t, b_t)) break;
-      }
-      if (have && it > 0) frag_store(x, A.Dl, j, ld, tm);
-      cg_iters += it;
-      return true;
-    }
-    // Rows in memory (a team owns several): the matrix is row-local, so s = H p and w = H r are
-    // formed from p and r in the pass instead of being carried (s = w + beta s) in two more
-    // arrays; a CG step reads r, p, x and W and writes r, p and x (7 arrays instead of 11).
-    // In exact arithmetic these are the iterates of the recurrence above.
-    // (Two rows per trip, their loads issued together, measured slower on the 2048^2 torus:
-    // the second row's fragments went to local memory.)
-    while (go && it < prm.cg_max_iter) {
-      double z[2] = {0.0, 0.0};
-      for (int j = tm.id; j < n; j += tm.count) {
-        Frag<T> r, pp, x, Wjt;
-        T aj = T(0);
-        cg7_load(j, it > 0, r, pp, x, Wjt, aj, Wt, ra);
-        cg7_step(j, r, pp, x, Wjt, aj, a_t, b_t, rho_t, gamma_t, z);
-      }
-      if (!sc.reduce(z, 2)) return false;
-      ++hess;
-      ++it;
-      if (!cg_scalars(lead, shs, z, target2, gam, ga, go, a_t, b_t)) break;
-    }
-    cg_iters += it;
-    return true;
-  }
-
-  // the Chronopoulos-Gear scalars after a reduction z = (r.r, w.r): thread 0 of the CTA
-  // evaluates them (one division) and shares them through shared memory; false when the
-  // CG stops (converged, a non-positive denominator, or NaN, which sets the status)
-  template <typename S>
-  __device__ __forceinline__ bool cg_scalars(bool lead, double* shs, const double* z,
-                                             double target2, double& gam, double& ga, int& go,
-                                             S& a_t, S& b_t) {
-    if (lead) {
-      int state = 0;                 // 0: go on, 1: stop, 2: NaN
-      const double gam_new = z[0], del_new = z[1];
+    T a_t, b_t;
+    bool go = cg_take(a_t, b_t) == 0;
+    // the scalars that follow from a reduction (r.r, w.r), in thread 0
+    auto scalars = [this](double gam_new, double del_new) {
+      double& gam = sc.scratch()[12];
+      double& ga = sc.scratch()[13];
+      const double target2 = sc.scratch()[14];
+      int state = 0;
       double alpha = 0.0, beta = 0.0;
       if (!(gam_new == gam_new) || !(del_new == del_new)) {
         state = 2;
@@ -1423,18 +1400,92 @@ struct Solver {
           state = 1;                     // rounding made the denominator non-positive
         }
       }
-      shs[0] = (double)state;
-      shs[1] = alpha;
-      shs[2] = beta;
+      cg_leave(state, alpha, beta);
+    };
+    it = 0;
+    if (tm.count >= n) {
+      // at most one row per team: its CG state stays in registers across the iterations
+      // (same arithmetic in the same order as below), and only delta is stored at the end, with
+      // a barrier before the neighbours read it; the iterations exchange nothing but their sums
+      const TeamRows row(this->tm, n);
+      const Team& tm = row.t;
+      const int j = row.j;
+      const bool have = row.more();      // the warp has a row (teams without one hold zeros)
+      Frag<T> r, w, pp, ss, x, Wjt;
+      frag_zero(pp);
+      frag_zero(ss);
+      frag_zero(x);
+      frag_load(r, A.R, j, ld, tm);
+      frag_load(w, A.HP, j, ld, tm);
+      frag_load(Wjt, Wt, j, ld, tm);
+      const T aj = ra[j];
+      while (go && it < prm.cg_max_iter) {
+        double z0 = 0.0, z1 = 0.0;
+        if (have) {
+#pragma unroll
+          for (int k = 0; k < KMAX; ++k)
+#pragma unroll
+            for (int e = 0; e < CHUNK; ++e) {
+              pp.v[k][e] = fma(b_t, pp.v[k][e], r.v[k][e]);
+              ss.v[k][e] = fma(b_t, ss.v[k][e], w.v[k][e]);
+              x.v[k][e] = fma(a_t, pp.v[k][e], x.v[k][e]);
+              r.v[k][e] = fma(-a_t, ss.v[k][e], r.v[k][e]);
+            }
+          local_h(r, Wjt, aj, rho_t, gamma_t, tm, w);
+          const T d1 = frag_dot(r, r, tm), d2 = frag_dot(w, r, tm);
+          pair_add(d1, d2, tm, z0, z1);
+        }
+        if (!sc.template reduce_pair<false>(z0, z1, tm.G, scalars)) return false;
+        ++hess;
+        ++it;
+        go = cg_take(a_t, b_t) == 0;
+      }
+      cg_iters += it;
+      if (it == 0) return true;
+      frag_store(x, A.Dl, j, ld, tm);
+      return sc.sync();
     }
-    __syncthreads();
-    const int state = (int)shs[0];
-    a_t = (S)shs[1];
-    b_t = (S)shs[2];
-    __syncthreads();
+    // Rows in memory (a team owns several): the matrix is row-local, so s = H p and w = H r are
+    // formed from p and r in the pass instead of being carried (s = w + beta s) in two more
+    // arrays; a CG step reads r, p, x and W and writes r, p and x (7 arrays instead of 11).
+    // In exact arithmetic these are the iterates of the recurrence above.
+    // (Two rows per trip, their loads issued together, measured slower on the 2048^2 torus:
+    // the second row's fragments went to local memory.)
+    while (go && it < prm.cg_max_iter) {
+      double z0 = 0.0, z1 = 0.0;
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
+        Frag<T> r, pp, x, Wjt;
+        T aj = T(0);
+        cg7_load(j, it > 0, r, pp, x, Wjt, aj, Wt, ra, tm);
+        cg7_step(j, r, pp, x, Wjt, aj, a_t, b_t, rho_t, gamma_t, tm, z0, z1);
+      }
+      if (!sc.template reduce_pair<true>(z0, z1, tm.G, scalars)) return false;
+      ++hess;
+      ++it;
+      go = cg_take(a_t, b_t) == 0;
+    }
+    cg_iters += it;
+    return true;
+  }
+
+  // What thread 0 of a CTA leaves for its threads after a reduction of a CG: the state (0 go on,
+  // 1 stop, 2 NaN, 3 the last step) and the scalars alpha and beta, rounded to T once.  The next
+  // reduction's first barrier separates the threads' reads from the next write.
+  __device__ __forceinline__ void cg_leave(int state, double alpha, double beta) const {
+    double* shs = sc.scratch() + 4;
+    reinterpret_cast<int*>(shs)[0] = state;
+    reinterpret_cast<T*>(shs + 1)[0] = (T)alpha;
+    reinterpret_cast<T*>(shs + 2)[0] = (T)beta;
+  }
+  __device__ __forceinline__ int cg_take(T& a_t, T& b_t) {
+    const double* shs = sc.scratch() + 4;
+    const int state = reinterpret_cast<const int*>(shs)[0];
+    a_t = reinterpret_cast<const T*>(shs + 1)[0];
+    b_t = reinterpret_cast<const T*>(shs + 2)[0];
     if (state == 2) status = ST_NAN;
-    go = state == 0;
-    return state == 0;
+    return state;
   }
 
   __device__ bool phase2_local(double rho, double& rho_out) {
@@ -1451,7 +1502,9 @@ struct Solver {
       if (status != ST_OK) break;
       // U^{k+1} = V^k + delta, -(C U^{k+1}), and the V-step's R_0 (W = U^{k+1})
       g3[0] = g3[1] = g3[2] = 0.0;
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         const RowCon c = row_con_of(j);
         Frag<double> Wj, Xj, mCW, mCX;
         Frag<T> Xt;
@@ -1468,12 +1521,12 @@ struct Solver {
           frag_axpy(Xt, T(1), x);                 // shadow of U^{k+1} = shadow(V^k) + delta
         }
         if (exact) frag_convert(Xt, Xj);          // re-rounded from the master every 32
-        local_mcx_row(j, A.V, A.Dl, it > 0, exact, mCW, mCX);
+        local_mcx_row(j, A.V, A.Dl, it > 0, exact, mCW, tm, mCX);
         frag_store(Xj, A.U, j, ld, tm);
         if (shadow) frag_store(Xt, A.Ut, j, ld, tm);
         frag_store(mCX, A.CWn, j, ld, tm);
-        const double qU = local_r0_row(j, Xj, Xt, mCX, c, c.lam, rho, gamma, g3);
-        if (c.i >= 0 && tm.lane == 0) A.e[c.i] = qU;  // a ||U_j^{k+1}||^2 for the output residual
+        const double qU = local_r0_row(j, Xj, Xt, mCX, c, c.lam, rho, gamma, tm, g3);
+        if (c.i >= 0 && tm.lead) A.e[c.i] = qU;  // a ||U_j^{k+1}||^2 for the output residual
       }
       if (!sc.reduce(g3, 3)) return false;
       ++hess;
@@ -1484,7 +1537,9 @@ struct Solver {
       const double rho_next =
           ((k + 1) % prm.rho_every == 0) ? fmin(rho * prm.rho_growth, prm.rho_max) : rho;
       double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         const RowCon c = row_con_of(j);
         const double qU = c.i >= 0 ? A.e[c.i] : 0.0;   // a ||U_j^{k+1}||^2 from pass A
         Frag<double> Wj, Xj, mCW, mCX;
@@ -1511,20 +1566,21 @@ struct Solver {
         if (exact) frag_convert(Xt, Xj);          // re-rounded from the master every 32
         // dual step lambda_i += rho (a U_j.V_j - b_i)
         double e = 0.0, lam_new = 0.0;
+        const double wx = frag_dot(Wj, Xj, tm);
         if (c.i >= 0) {
-          e = c.a * frag_dot(Wj, Xj, tm) - c.b;
+          e = c.a * wx - c.b;
           lam_new = c.lam + rho * e;        // every lane of the team holds the same value
         }
-        local_mcx_row(j, A.U, A.Dl, it > 0, exact, mCW, mCX);
+        local_mcx_row(j, A.U, A.Dl, it > 0, exact, mCW, tm, mCX);
         frag_store(Xj, A.V, j, ld, tm);
         if (shadow) frag_store(Xt, A.Vt, j, ld, tm);
         frag_store(mCX, A.CWn, j, ld, tm);
-        const double qV = local_r0_row(j, Xj, Xt, mCX, c, lam_new, rho_next, gamma, v + 5);
+        const double qV = local_r0_row(j, Xj, Xt, mCX, c, lam_new, rho_next, gamma, tm, v + 5);
         // the output's row residual a ||(U_j + V_j)/2||^2 - b_i from a||U_j||^2 (pass A),
         // a U_j.V_j = e + b_i and a||V_j||^2
         double eh = 0.0;
         if (c.i >= 0) eh = 0.25 * (qU + 2.0 * (e + c.b) + qV) - c.b;
-        if (tm.lane == 0) {
+        if (tm.lead) {
           if (c.i >= 0) A.lam[c.i] = lam_new;
           v[0] += e * e;
           v[1] += eh * eh;
@@ -1592,7 +1648,9 @@ struct Solver {
     for (int k = admm_iters; k < prm.max_admm_iter; ++k) {
       const bool exact = (k + 1) % 32 == 0;
       // pass A: U-step finish and the V-step's solution
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         const RowCon c = row_con_of(j);
         Frag<double> Wj, Xj, mCW, mCX, xd;
         Frag<T> Xt, x;
@@ -1605,12 +1663,12 @@ struct Solver {
         frag_axpy(Xj, 1.0, xd);
         frag_axpy(Xt, T(1), x);                   // shadow of U^{k+1} = shadow(V^k) + delta
         if (exact) frag_convert(Xt, Xj);          // re-rounded from the master every 32
-        local_mcx_row(j, A.V, dU, true, exact, mCW, mCX);
+        local_mcx_row(j, A.V, dU, true, exact, mCW, tm, mCX);
         frag_store(Xj, A.U, j, ld, tm);
         if (shadow) frag_store(Xt, A.Ut, j, ld, tm);
         frag_store(mCX, A.CWn, j, ld, tm);
-        const double qU = local_r0_row(j, Xj, Xt, mCX, c, c.lam, rho, gamma, g3, dV);
-        if (c.i >= 0 && tm.lane == 0) A.e[c.i] = qU;  // a ||U_j^{k+1}||^2 for the output residual
+        const double qU = local_r0_row(j, Xj, Xt, mCX, c, c.lam, rho, gamma, tm, g3, dV);
+        if (c.i >= 0 && tm.lead) A.e[c.i] = qU;  // a ||U_j^{k+1}||^2 for the output residual
       }
       if (!sc.sync()) return false;
       ++hess;
@@ -1618,7 +1676,9 @@ struct Solver {
       const double rho_next =
           ((k + 1) % prm.rho_every == 0) ? fmin(rho * prm.rho_growth, prm.rho_max) : rho;
       double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         const RowCon c = row_con_of(j);
         const double qU = c.i >= 0 ? A.e[c.i] : 0.0;   // a ||U_j^{k+1}||^2 from pass A
         Frag<double> Wj, Xj, mCW, mCX, xd;
@@ -1640,20 +1700,21 @@ struct Solver {
         if (exact) frag_convert(Xt, Xj);          // re-rounded from the master every 32
         // dual step lambda_i += rho (a U_j.V_j - b_i)
         double e = 0.0, lam_new = 0.0;
+        const double wx = frag_dot(Wj, Xj, tm);
         if (c.i >= 0) {
-          e = c.a * frag_dot(Wj, Xj, tm) - c.b;
+          e = c.a * wx - c.b;
           lam_new = c.lam + rho * e;        // every lane of the team holds the same value
         }
-        local_mcx_row(j, A.U, dV, true, exact, mCW, mCX);
+        local_mcx_row(j, A.U, dV, true, exact, mCW, tm, mCX);
         frag_store(Xj, A.V, j, ld, tm);
         if (shadow) frag_store(Xt, A.Vt, j, ld, tm);
         frag_store(mCX, A.CWn, j, ld, tm);
-        const double qV = local_r0_row(j, Xj, Xt, mCX, c, lam_new, rho_next, gamma, g3, dU);
+        const double qV = local_r0_row(j, Xj, Xt, mCX, c, lam_new, rho_next, gamma, tm, g3, dU);
         // the output's row residual a ||(U_j + V_j)/2||^2 - b_i from a||U_j||^2 (pass A),
         // a U_j.V_j = e + b_i and a||V_j||^2
         double eh = 0.0;
         if (c.i >= 0) eh = 0.25 * (qU + 2.0 * (e + c.b) + qV) - c.b;
-        if (tm.lane == 0) {
+        if (tm.lead) {
           if (c.i >= 0) A.lam[c.i] = lam_new;
           v[0] += e * e;
           v[1] += eh * eh;
@@ -1722,7 +1783,7 @@ struct Solver {
   // (H Z)_j for the tangent field Z (neighbours' rows of Z must be visible); Zj is row j of Z,
   // Uj row j of the iterate; in T (the CG of a Newton step runs in the form's element type)
   __device__ __forceinline__ void sphere_hess_row(int j, const T* Z, const Frag<T>& Zj,
-                                                  const Frag<T>& Uj, T u2, T mu,
+                                                  const Frag<T>& Uj, T u2, T mu, const Team& tm,
                                                   Frag<T>& out) const {
     Frag<T> mCZ;
     spmm_row<T>(P, Z, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, T(0), tm, mCZ);
@@ -1741,7 +1802,9 @@ struct Solver {
   // g, mu, lambda(U) and C U at the iterate in A.U; v = (||g||^2, <C, U U^T>, ||U||_F^2, time)
   __device__ bool sphere_gradient(double* v) {
     v[0] = v[1] = v[2] = v[3] = 0.0;
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> Uj, mCU, g;
       frag_load(Uj, A.U, j, ld, tm);
       spmm_row<double>(P, A.U, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, 0.0, tm, mCU);
@@ -1754,7 +1817,7 @@ struct Solver {
         for (int e = 0; e < CHUNK; ++e) g.v[k][e] = 2.0 * (-mCU.v[k][e] - mu * Uj.v[k][e]);
       frag_store(g, A.grad, j, ld, tm);
       const double g2 = frag_dot(g, g, tm);
-      if (tm.lane == 0) {
+      if (tm.lead) {
         A.e[j] = mu;
         const int ci = P.row_con[j];
         A.lam[ci] = -mu / P.row_a[j];
@@ -1775,7 +1838,8 @@ struct Solver {
   // *c buffers, written to the *n ones) and one barrier per CG step remains, the reduction.
   __device__ __forceinline__ void sphere_tcg_row(int j, const T* Rc, const T* Wc, const T* Sc,
                                                  T* Rn, T* Wn, T* Sn, T a_t, T b_t, bool have_ps,
-                                                 bool want_h, double* z) {
+                                                 bool want_h, const Team& tm, double& z0,
+                                                 double& z1) {
     Frag<T> r, w, pd, ss, x;
     frag_load(r, Rc, j, ld, tm);
     frag_load(w, Wc, j, ld, tm);
@@ -1841,11 +1905,8 @@ struct Solver {
 #pragma unroll
       for (int e = 0; e < CHUNK; ++e) acc.v[k][e] = T(2) * (acc.v[k][e] - cp * Uj.v[k][e]);
     frag_store(acc, Wn, j, ld, tm);
-    const double d1 = (double)frag_dot(r, r, tm), d2 = (double)frag_dot(acc, r, tm);
-    if (tm.lane == 0) {
-      z[0] += d1;
-      z[1] += d2;
-    }
+    const T d1 = frag_dot(r, r, tm), d2 = frag_dot(acc, r, tm);
+    pair_add(d1, d2, tm, z0, z1);
   }
 
   // Steihaug-Toint truncated CG (Absil, Mahony and Sepulchre 2008, Algorithm 11) for the
@@ -1864,7 +1925,9 @@ struct Solver {
     T* Sb[2] = {A.Sv, reinterpret_cast<T*>(A.dir)};
     const T* const Us = A.Ut;
     // r_0 = -g, w_0 = H r_0
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> gj;
       Frag<T> r;
       frag_load(gj, A.grad, j, ld, tm);
@@ -1877,32 +1940,31 @@ struct Solver {
     }
     if (!sc.sync()) return false;
     double g3[2] = {0.0, 0.0};
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<T> Uj, r, w;
       frag_load(Uj, Us, j, ld, tm);
       frag_load(r, Rb[0], j, ld, tm);
       const T u2 = frag_dot(Uj, Uj, tm);
-      sphere_hess_row(j, Rb[0], r, Uj, u2, (T)A.e[j], w);
+      sphere_hess_row(j, Rb[0], r, Uj, u2, (T)A.e[j], tm, w);
       frag_store(w, Wb[0], j, ld, tm);
       const double d1 = (double)frag_dot(r, r, tm), d2 = (double)frag_dot(w, r, tm);
-      if (tm.lane == 0) {
+      if (tm.lead) {
         g3[0] += d1;
         g3[1] += d2;
       }
     }
     if (!sc.reduce(g3, 2)) return false;
-    const bool lead = threadIdx.x == 0;
-    double* shs = sc.scratch() + 4;     // state (0 go on, 1 stop, 2 NaN, 3 last step), a, b
     const double eta = fmin(0.5, sqrt(sqrt(g2)));
     const double target2 = eta * eta * g2;
     const double dl2 = delta * delta;
     // thread 0: gam = r.r, ga = gam * alpha, a_prev = alpha, pp = ||p||^2, dp = d.p,
     // dd = ||d||^2 (of the direction / iterate the next pass forms)
-    double gam = 0.0, ga = 0.0, a_prev = 0.0, pp = 0.0, dp = 0.0, dd = 0.0;
-    if (lead) {
-      gam = g3[0];
-      const double del = g3[1];
-      pp = gam;
+    // (in shared memory, see cg_local_loop)
+    double* const own = sc.scratch() + 12;
+    if (threadIdx.x == 0) {
+      const double gam = g3[0], del = g3[1];
       int state = 0;
       double alpha = 0.0;
       if (!(gam == gam) || !(del == del)) {
@@ -1915,17 +1977,67 @@ struct Solver {
       } else {
         alpha = gam / del;
       }
-      ga = gam * alpha;
-      a_prev = alpha;
-      shs[0] = (double)state;
-      shs[1] = alpha;
-      shs[2] = 0.0;
+      own[0] = gam;
+      own[1] = gam * alpha;
+      own[2] = alpha;
+      own[3] = gam;
+      own[4] = 0.0;
+      own[5] = 0.0;
+      own[6] = target2;
+      own[7] = dl2;
+      cg_leave(state, alpha, 0.0);
     }
     __syncthreads();
-    int state = (int)shs[0];
-    T a_t = (T)shs[1], b_t = T(0);
-    __syncthreads();
-    if (state == 2) status = ST_NAN;
+    T a_t, b_t;
+    int state = cg_take(a_t, b_t);
+    // the scalars that follow from a reduction (r.r, w.r), in thread 0
+    auto scalars = [this, own](double gam_new, double del_new) {
+      double gam = own[0], ga = own[1], a_prev = own[2], pp = own[3], dp = own[4], dd = own[5];
+      const double target2 = own[6], dl2 = own[7];
+      // the pass just made: d += alpha p (the alpha of the previous step), so d.p and ||d||^2
+      // move on
+      const double alpha_prev = a_prev;
+      dd += 2.0 * alpha_prev * dp + alpha_prev * alpha_prev * pp;
+      dp += alpha_prev * pp;           // d_k+1 . p_k
+      int st = 0;
+      double alpha = 0.0, beta = 0.0;
+      if (!(gam_new == gam_new) || !(del_new == del_new)) {
+        st = 2;
+      } else if (gam_new <= target2) {
+        st = 1;
+      } else {
+        // with D = del_new ga - gam_new^2 (p.Hp = D / ga), beta = gam_new / gam and
+        // alpha = gam_new ga / D both come from the one reciprocal 1 / (gam D) when D > 0
+        const double D = del_new * ga - gam_new * gam_new;
+        bool to_boundary = !(D > 0.0);
+        if (!to_boundary) {
+          const double inv = 1.0 / (gam * D);
+          beta = gam_new * D * inv;
+          alpha = gam_new * ga * gam * inv;
+        } else {
+          beta = gam_new / gam;
+        }
+        pp = gam_new + beta * beta * pp;          // ||p_k+1||^2
+        dp = beta * dp;                           // d_k+1 . p_k+1
+        if (!to_boundary)
+          to_boundary = dd + 2.0 * alpha * dp + alpha * alpha * pp >= dl2;
+        if (to_boundary) {
+          const double qa = pp, qb = 2.0 * dp, qc = dd - dl2;
+          alpha = (-qb + sqrt(fmax(qb * qb - 4.0 * qa * qc, 0.0))) / (2.0 * qa);
+          st = 3;
+        }
+        ga = gam_new * alpha;
+        gam = gam_new;
+        a_prev = alpha;
+      }
+      cg_leave(st, alpha, beta);
+      own[0] = gam;
+      own[1] = ga;
+      own[2] = a_prev;
+      own[3] = pp;
+      own[4] = dp;
+      own[5] = dd;
+    };
     it = 0;
     on_boundary = state == 3;
     bool wrote = false;
@@ -1935,84 +2047,38 @@ struct Solver {
     constexpr bool fuse = sizeof(T) == 4;
     while ((state == 0 || state == 3) && it < prm.newton_cg_max) {
       const bool want_h = state == 0;
-      double z[2] = {0.0, 0.0};
-      for (int j = tm.id; j < n; j += tm.count)
-        sphere_tcg_row(j, Rb[cur], Wb[cur], Sb[cur], Rb[cur ^ 1], Wb[cur ^ 1], Sb[cur ^ 1], a_t,
-                       b_t, wrote, want_h && fuse, z);
+      double z0 = 0.0, z1 = 0.0;
+      for (TeamRows rows(tm, n); rows.more(); rows.next())
+        sphere_tcg_row(rows.j, Rb[cur], Wb[cur], Sb[cur], Rb[cur ^ 1], Wb[cur ^ 1], Sb[cur ^ 1],
+                       a_t, b_t, wrote, want_h && fuse, rows.t, z0, z1);
       wrote = true;
       cur ^= 1;
       if (!want_h) break;                // the boundary step: d is final
       if (!fuse) {
         if (!sc.sync()) return false;
-        for (int j = tm.id; j < n; j += tm.count) {
+        for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+          const Team& tm = rows.t;
+          const int j = rows.j;
           Frag<T> Uj, r, w;
           frag_load(Uj, Us, j, ld, tm);
           frag_load(r, Rb[cur], j, ld, tm);
           const T u2 = frag_dot(Uj, Uj, tm);
-          sphere_hess_row(j, Rb[cur], r, Uj, u2, (T)A.e[j], w);
+          sphere_hess_row(j, Rb[cur], r, Uj, u2, (T)A.e[j], tm, w);
           frag_store(w, Wb[cur], j, ld, tm);
-          const double d1 = (double)frag_dot(r, r, tm), d2 = (double)frag_dot(w, r, tm);
-          if (tm.lane == 0) {
-            z[0] += d1;
-            z[1] += d2;
-          }
+          const T d1 = frag_dot(r, r, tm), d2 = frag_dot(w, r, tm);
+          pair_add(d1, d2, tm, z0, z1);
         }
       }
-      if (!sc.reduce(z, 2)) return false;
+      if (!sc.template reduce_pair<true>(z0, z1, tm.G, scalars)) return false;
       ++it;
-      if (lead) {
-        // the pass just made: d += alpha p (the alpha of the previous step), so d.p and ||d||^2
-        // move on
-        const double alpha_prev = a_prev;
-        dd += 2.0 * alpha_prev * dp + alpha_prev * alpha_prev * pp;
-        dp += alpha_prev * pp;           // d_k+1 . p_k
-        const double gam_new = z[0], del_new = z[1];
-        int st = 0;
-        double alpha = 0.0, beta = 0.0;
-        if (!(gam_new == gam_new) || !(del_new == del_new)) {
-          st = 2;
-        } else if (gam_new <= target2) {
-          st = 1;
-        } else {
-          // with D = del_new ga - gam_new^2 (p.Hp = D / ga), beta = gam_new / gam and
-          // alpha = gam_new ga / D both come from the one reciprocal 1 / (gam D) when D > 0
-          const double D = del_new * ga - gam_new * gam_new;
-          bool to_boundary = !(D > 0.0);
-          if (!to_boundary) {
-            const double inv = 1.0 / (gam * D);
-            beta = gam_new * D * inv;
-            alpha = gam_new * ga * gam * inv;
-          } else {
-            beta = gam_new / gam;
-          }
-          pp = gam_new + beta * beta * pp;          // ||p_k+1||^2
-          dp = beta * dp;                           // d_k+1 . p_k+1
-          if (!to_boundary)
-            to_boundary = dd + 2.0 * alpha * dp + alpha * alpha * pp >= dl2;
-          if (to_boundary) {
-            const double qa = pp, qb = 2.0 * dp, qc = dd - dl2;
-            alpha = (-qb + sqrt(fmax(qb * qb - 4.0 * qa * qc, 0.0))) / (2.0 * qa);
-            st = 3;
-          }
-          ga = gam_new * alpha;
-          gam = gam_new;
-          a_prev = alpha;
-        }
-        shs[0] = (double)st;
-        shs[1] = alpha;
-        shs[2] = beta;
-      }
-      __syncthreads();
-      state = (int)shs[0];
-      a_t = (T)shs[1];
-      b_t = (T)shs[2];
-      __syncthreads();
-      if (state == 2) status = ST_NAN;
+      state = cg_take(a_t, b_t);
       if (state == 3) on_boundary = true;
     }
     if (!wrote) {
       // no step taken (the gradient already small, or a NaN): d = 0
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<T> x;
         frag_zero(x);
         frag_store(x, A.Dl, j, ld, tm);
@@ -2024,17 +2090,19 @@ struct Solver {
   // the model's decrease -(g.d + d.H d / 2) for the d in A.Dl (neighbours' d visible)
   __device__ bool sphere_model_decrease(double& pred) {
     double v[2] = {0.0, 0.0};
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<T> Uj, dj, w;
       Frag<double> gj, dd;
       frag_load(Uj, A.Ut, j, ld, tm);
       frag_load(dj, A.Dl, j, ld, tm);
       const T u2 = frag_dot(Uj, Uj, tm);
-      sphere_hess_row(j, A.Dl, dj, Uj, u2, (T)A.e[j], w);
+      sphere_hess_row(j, A.Dl, dj, Uj, u2, (T)A.e[j], tm, w);
       frag_load(gj, A.grad, j, ld, tm);
       frag_convert(dd, dj);
       const double a1 = frag_dot(gj, dd, tm), a2 = (double)frag_dot(dj, w, tm);
-      if (tm.lane == 0) {
+      if (tm.lead) {
         v[0] += a1;
         v[1] += a2;
       }
@@ -2047,7 +2115,9 @@ struct Solver {
   // trial point R(U + t d) into A.V (row scaling onto the spheres); with want_slope also g.d
   __device__ bool sphere_trial(double t, bool want_slope, double& slope) {
     double v[1] = {0.0};
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> Uj, dj;
       Frag<T> dt;
       frag_load(Uj, A.U, j, ld, tm);
@@ -2057,7 +2127,7 @@ struct Solver {
         Frag<double> gj;
         frag_load(gj, A.grad, j, ld, tm);
         const double gd = frag_dot(gj, dj, tm);
-        if (tm.lane == 0) v[0] += gd;
+        if (tm.lead) v[0] += gd;
       }
       frag_axpy(Uj, t, dj);
       const double sc2 = P.row_norm[j] / sqrt(frag_dot(Uj, Uj, tm));
@@ -2075,12 +2145,14 @@ struct Solver {
   // <C, W W^T> for W = A.V (neighbours visible)
   __device__ bool trial_objective(double& f) {
     double v[1] = {0.0};
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> Wj, mCW;
       frag_load(Wj, A.V, j, ld, tm);
       spmm_row<double>(P, A.V, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, 0.0, tm, mCW);
       const double o = -frag_dot(Wj, mCW, tm);
-      if (tm.lane == 0) v[0] += o;
+      if (tm.lead) v[0] += o;
     }
     if (!sc.reduce(v, 1)) return false;
     f = v[0];
@@ -2092,7 +2164,9 @@ struct Solver {
   __device__ bool copy_rows(const double* src, double* dst, T* tdst = nullptr) {
     const bool sh = tdst != nullptr && (const void*)tdst != (const void*)A.U &&
                     (const void*)tdst != (const void*)A.V;
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> x;
       frag_load(x, src, j, ld, tm);
       frag_store(x, dst, j, ld, tm);
@@ -2109,7 +2183,9 @@ struct Solver {
   // T shadow of U
   __device__ bool sphere_retract_u() {
     const bool sh = (const void*)A.Ut != (const void*)A.U;
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> Uj;
       frag_load(Uj, A.U, j, ld, tm);
       const double sc2 = P.row_norm[j] / sqrt(frag_dot(Uj, Uj, tm));
@@ -2181,11 +2257,13 @@ struct Solver {
   // ||U||_F^2 of the masters
   __device__ bool u_norm2(double& u2) {
     double v[1] = {0.0};
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> Uj;
       frag_load(Uj, A.U, j, ld, tm);
       const double d = frag_dot(Uj, Uj, tm);
-      if (tm.lane == 0) v[0] += d;
+      if (tm.lead) v[0] += d;
     }
     if (!sc.reduce(v, 1)) return false;
     u2 = v[0];
@@ -2235,7 +2313,9 @@ struct Solver {
 
   // U_hat = (U + V)/2 into tmp
   __device__ bool form_u_hat() {
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> u, w;
       frag_load(u, A.U, j, ld, tm);
       frag_load(w, A.V, j, ld, tm);
@@ -2258,7 +2338,9 @@ struct Solver {
     if (!form_u_hat()) return false;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     if (P.a_diag_only) {
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<double> Uh, mCU;
         frag_load(Uh, A.tmp, j, ld, tm);
         spmm_row<double>(P, A.tmp, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, 0.0, tm, mCU);
@@ -2267,7 +2349,7 @@ struct Solver {
         const int ci = P.row_con[j];
         if (ci >= 0) frag_axpy(mCU, -P.row_a[j] * A.lam[ci], Uh);
         const double s2 = frag_dot(mCU, mCU, tm);
-        if (tm.lane == 0) {
+        if (tm.lead) {
           v[0] += o;
           v[2] += u2;
           v[3] += s2;
@@ -2280,14 +2362,12 @@ struct Solver {
         frag_load(Uh, A.tmp, j, ld, wr.st);
         spmm_row_warp<double>(P, A.tmp, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, 0.0, wr, mCU);
         spmm_row_warp<double>(P, A.tmp, ld, j, A.lam, nullptr, 0.0, -1.0, 0.0, 0.0, wr, mSU);
-        if (wr.sub == 0) {
-          const double o = -frag_dot(Uh, mCU, wr.st), u2 = frag_dot(Uh, Uh, wr.st);
-          const double s2 = frag_dot(mSU, mSU, wr.st);
-          if (wr.st.lane == 0) {
-            v[0] += o;
-            v[2] += u2;
-            v[3] += s2;
-          }
+        const double o = -frag_dot(Uh, mCU, wr.st), u2 = frag_dot(Uh, Uh, wr.st);
+        const double s2 = frag_dot(mSU, mSU, wr.st);
+        if (wr.sub == 0 && wr.st.lead) {
+          v[0] += o;
+          v[2] += u2;
+          v[3] += s2;
         }
       }
     }
@@ -2721,7 +2801,9 @@ struct Solver {
     set_rank(r_new);
     const double tau = zn2 > 0.0 ? prm.escape_scale * sqrt(uh_norm2 / (double)r_old / zn2) : 0.0;
     const bool shadow = (const void*)A.Ut != (const void*)A.U;
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> u, w;
       const double zj = tau * zv[j];
 #pragma unroll
@@ -2755,13 +2837,15 @@ struct Solver {
     if (!form_u_hat()) return false;
     double v[6] = {0, 0, 0, 0, 0, 0};
     if (P.a_diag_only) {
-      for (int j = tm.id; j < n; j += tm.count) {
+      for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+        const Team& tm = rows.t;
+        const int j = rows.j;
         Frag<double> Uh, mCU, mSU;
         frag_load(Uh, A.tmp, j, ld, tm);
         spmm_row<double>(P, A.tmp, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, 0.0, tm, mCU);
         spmm_row<double>(P, A.tmp, ld, j, A.lam, nullptr, 0.0, -1.0, 0.0, 0.0, tm, mSU);
         const double o = -frag_dot(Uh, mCU, tm), d = frag_dot(mSU, mSU, tm);
-        if (tm.lane == 0) {
+        if (tm.lead) {
           v[0] += o;
           v[1] += d;
         }
@@ -2773,12 +2857,10 @@ struct Solver {
         frag_load(Uh, A.tmp, j, ld, wr.st);
         spmm_row_warp<double>(P, A.tmp, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, 0.0, wr, mCU);
         spmm_row_warp<double>(P, A.tmp, ld, j, A.lam, nullptr, 0.0, -1.0, 0.0, 0.0, wr, mSU);
-        if (wr.sub == 0) {
-          const double o = -frag_dot(Uh, mCU, wr.st), d = frag_dot(mSU, mSU, wr.st);
-          if (wr.st.lane == 0) {
-            v[0] += o;
-            v[1] += d;
-          }
+        const double o = -frag_dot(Uh, mCU, wr.st), d = frag_dot(mSU, mSU, wr.st);
+        if (wr.sub == 0 && wr.st.lead) {
+          v[0] += o;
+          v[1] += d;
         }
       }
     }
@@ -2789,17 +2871,19 @@ struct Solver {
       v[4] += es * es;
     };
     if (P.a_multi) {
-      if (!con_chunks<2>([&](int r, int c, double a, double* s) {
-            s[0] += sddmm_entry<double>(A.tmp, A.tmp, ld, r, c, a, tmc);
-            s[1] += sddmm_entry<double>(A.U, A.V, ld, r, c, a, tmc);
+      if (!con_chunks<2>([&](int r, int c, double a, const Team& tmc, double* s) {
+            s[0] = sddmm_entry<double>(A.tmp, A.tmp, ld, r, c, a, tmc);
+            s[1] = sddmm_entry<double>(A.U, A.V, ld, r, c, a, tmc);
           }))
         return false;
       for (int i = sc.tid(); i < m; i += sc.nthreads()) add(i, con_total(i, 0), con_total(i, 1));
     } else {
-      for (int i = tmc.id; i < m; i += tmc.count) {
+      for (TeamRows rows(this->tmc, m); rows.more(); rows.next()) {
+        const Team& tmc = rows.t;
+        const int i = rows.j;
         const double q = sddmm_con<double>(P, A.tmp, A.tmp, ld, i, tmc);
         const double qs = sddmm_con<double>(P, A.U, A.V, ld, i, tmc);
-        if (tmc.lane == 0) add(i, q, qs);
+        if (tmc.lead) add(i, q, qs);
       }
     }
     if (!sc.reduce(v, 5)) return false;
@@ -2832,7 +2916,9 @@ struct Solver {
       }
     }
     // switch: V = U (Algorithm 2), or the checkpointed V of a resume; shadows
-    for (int j = tm.id; j < n; j += tm.count) {
+    for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
+      const Team& tm = rows.t;
+      const int j = rows.j;
       Frag<double> u, w;
       frag_load(u, A.U, j, ld, tm);
       if (prm.resume) frag_load(w, A.V, j, ld, tm);
