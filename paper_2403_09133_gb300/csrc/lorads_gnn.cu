@@ -9,6 +9,7 @@
 // Loss (rotation invariant): mean over edges of (U_i.U_j - Xs_ij)^2 + beta mean (y_i - ys_i)^2.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -50,8 +51,58 @@ struct GemmArgs {
   bf16* out_h;               // EPI_LAYER: H (BF16, ld CATW)
   const float* bias;         // EPI_LAYER: b (HID); EPI_HEADS: b_y at bias[0]
   float* partial;            // EPI_WGRAD: [tile][128][N]
+  double* bias_partial;      // EPI_WGRAD: [tile][N], the tile's column sums of B
   int* err;
 };
+
+// An operand tile of R rows x K columns, K-major in shared memory, whose source is stored the
+// other way round: entry (row, k) is src[(node0 + k) * ld + row], zero past `rows` rows or `nodes`
+// nodes.  A thread moves blocks of 8 nodes x 8 rows: eight 16-byte loads (one per node), a
+// transpose in registers, eight 16-byte stores.  Loading the entries one by one (2 bytes every
+// ld) had the weight-gradient GEMM wait on 128 scattered loads per thread.
+template <int R, int K>
+__device__ __forceinline__ void stage_transposed(const bf16* src, int ld, int rows, int node0,
+                                                 int nodes, uint8_t* dst) {
+  for (int b = threadIdx.x; b < (R / 8) * (K / 8); b += 128) {
+    const int r0 = (b % (R / 8)) * 8, k0 = (b / (R / 8)) * 8;   // lanes along a node's row
+    uint4 in[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int node = node0 + k0 + e;
+      in[e] = (node < nodes && r0 < rows)
+                  ? *reinterpret_cast<const uint4*>(src + (size_t)node * ld + r0)
+                  : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      // row r0 + q: the q-th 16-bit entry of each of the eight nodes
+      uint32_t w[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const uint32_t* lo = reinterpret_cast<const uint32_t*>(&in[2 * e]);
+        const uint32_t* hi = reinterpret_cast<const uint32_t*>(&in[2 * e + 1]);
+        w[e] = __byte_perm(lo[q >> 1], hi[q >> 1], (q & 1) ? 0x7632 : 0x5410);
+      }
+      *reinterpret_cast<uint4*>(dst + tc::sw128_offset(r0 + q, k0, R)) =
+          make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+}
+
+// An operand tile stored K-major in the source too: entry (row, k) is src[(row0 + row) * ld + k],
+// zero past `rows` rows or `cols` columns
+template <int R, int K>
+__device__ __forceinline__ void stage_rows(const bf16* src, int ld, int row0, int rows, int cols,
+                                           uint8_t* dst) {
+  for (int idx = threadIdx.x; idx < R * (K / 8); idx += 128) {
+    const int m = idx / (K / 8), kc = (idx % (K / 8)) * 8;
+    const int row = row0 + m;
+    const uint4 v = (row < rows && kc < cols)
+                        ? *reinterpret_cast<const uint4*>(src + (size_t)row * ld + kc)
+                        : make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(dst + tc::sw128_offset(m, kc, R)) = v;
+  }
+}
 
 template <int N, int K>
 __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g) {
@@ -67,47 +118,10 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g) {
   const int row0 = tile * 128;
   if (warp == 0) tc::tmem_alloc(&tmem_base, N);
   if (tid == 0) tc::mbar_init(&bar, 1);
-  // A tile: 128 x K, K-major
-  for (int idx = tid; idx < 128 * (K / 8); idx += 128) {
-    const int m = idx / (K / 8), kc = (idx % (K / 8)) * 8;
-    __align__(16) bf16 v[8];
-    if (!g.a_trans) {
-      const int row = row0 + m;
-      if (row < g.rows && kc < g.a_cols) {
-        *reinterpret_cast<uint4*>(v) = *reinterpret_cast<const uint4*>(g.A + (size_t)row * g.lda + kc);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = __float2bfloat16(0.f);
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int node = row0 + kc + e;
-        v[e] = (node < g.rows && m < g.a_cols) ? g.A[(size_t)node * g.lda + m] : __float2bfloat16(0.f);
-      }
-    }
-    *reinterpret_cast<uint4*>(sA + tc::sw128_offset(m, kc, 128)) = *reinterpret_cast<uint4*>(v);
-  }
-  // B tile: N x K, K-major
-  for (int idx = tid; idx < N * (K / 8); idx += 128) {
-    const int nn = idx / (K / 8), kc = (idx % (K / 8)) * 8;
-    __align__(16) bf16 v[8];
-    if (!g.b_trans) {
-      if (nn < g.b_rows && kc < g.b_cols) {
-        *reinterpret_cast<uint4*>(v) = *reinterpret_cast<const uint4*>(g.B + (size_t)nn * g.ldb + kc);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = __float2bfloat16(0.f);
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int node = row0 + kc + e;
-        v[e] = (node < g.rows && nn < g.b_rows) ? g.B[(size_t)node * g.ldb + nn] : __float2bfloat16(0.f);
-      }
-    }
-    *reinterpret_cast<uint4*>(sB + tc::sw128_offset(nn, kc, N)) = *reinterpret_cast<uint4*>(v);
-  }
+  if (g.a_trans) stage_transposed<128, K>(g.A, g.lda, g.a_cols, row0, g.rows, sA);
+  else stage_rows<128, K>(g.A, g.lda, row0, g.rows, g.a_cols, sA);
+  if (g.b_trans) stage_transposed<N, K>(g.B, g.ldb, g.b_rows, row0, g.rows, sB);
+  else stage_rows<N, K>(g.B, g.ldb, 0, g.b_rows, g.b_cols, sB);
   tc::fence_proxy_async_smem();
   tc::fence_before();
   __syncthreads();
@@ -124,6 +138,25 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g) {
     }
     tc::mma_commit(&bar);
   }
+  if (g.epi == EPI_WGRAD) {
+    // the bias gradient: column sums of B (its rows here) over the tile's nodes, FP64, by 128 / N
+    // threads per column while the tensor core runs; combined in the partial sums' order
+    constexpr int PER = 128 / N, KP = K / PER;
+    const int c = tid / PER, part = tid % PER;
+    double bs = 0.0;
+    for (int k = part * KP; k < (part + 1) * KP; k += 8) {
+      const uint4 v = *reinterpret_cast<const uint4*>(sB + tc::sw128_offset(c, k, N));
+      const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        bs += (double)__bfloat162float(h[e].x);
+        bs += (double)__bfloat162float(h[e].y);
+      }
+    }
+#pragma unroll
+    for (int off = 1; off < PER; off <<= 1) bs += __shfl_xor_sync(0xffffffffu, bs, off);
+    if (part == 0) g.bias_partial[(size_t)tile * N + c] = bs;
+  }
   const bool ok = tc::mbar_wait(&bar, 0, 1LL << 24);
   if (!ok && lane == 0) atomicExch(g.err, 1);
   tc::fence_after();
@@ -136,7 +169,9 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g) {
     if (g.epi == EPI_WGRAD) {
       float* pp = g.partial + ((size_t)tile * 128 + m) * N + c0;
 #pragma unroll
-      for (int i = 0; i < 16; ++i) pp[i] = acc[i];
+      for (int i = 0; i < 16; i += 4)
+        *reinterpret_cast<float4*>(pp + i) =
+            make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
     } else if (row < g.rows) {
       if (g.epi == EPI_LAYER) {
 #pragma unroll
@@ -164,26 +199,39 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g) {
 
 template <int N, int K>
 static cudaError_t launch_gemm(const GemmArgs& g, int tiles, cudaStream_t s) {
-  const size_t smem = (size_t)128 * K * 2 + (size_t)N * K * 2 + 1024;
-  cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<N, K>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  constexpr size_t smem = (size_t)128 * K * 2 + (size_t)N * K * 2 + 1024;
+  if constexpr (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<N, K>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
   tc_gemm_kernel<N, K><<<tiles, 128, smem, s>>>(g);
   return cudaGetLastError();
 }
 
 // ---- features: z_i (8 normals), 1, log(1+deg), d/10, s, zeros ----
+// One thread per node and group of eight columns (group 0: one thread per normal number, whose FP64
+// logarithm and cosine are the work: 1/64 of the FP32 rate here, so they are spread over all SMs).
 __global__ void features_kernel(int n, const float* deg, const float* dsum, const float* ssum,
                                 unsigned long long key, bf16* cat0) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  const long long work = (long long)n * 16;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < work;
+       t += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(t >> 4), c = (int)(t & 15);
     bf16* row = cat0 + (size_t)i * CATW;
-    for (int c = 0; c < NRAND; ++c)
+    if (c < NRAND) {
       row[c] = __float2bfloat16((float)normal_at(key, (uint64_t)i * NRAND + c));
-    row[NRAND] = __float2bfloat16(1.f);
-    row[NRAND + 1] = __float2bfloat16(log1pf(deg[i]));
-    row[NRAND + 2] = __float2bfloat16(dsum[i] / 10.f);
-    row[NRAND + 3] = __float2bfloat16(ssum[i]);
-    for (int c = NRAND + 4; c < HID; ++c) row[c] = __float2bfloat16(0.f);
+    } else if (c == NRAND) {
+      // columns 8 .. 15
+      row[NRAND] = __float2bfloat16(1.f);
+      row[NRAND + 1] = __float2bfloat16(log1pf(deg[i]));
+      row[NRAND + 2] = __float2bfloat16(dsum[i] / 10.f);
+      row[NRAND + 3] = __float2bfloat16(ssum[i]);
+      *reinterpret_cast<uint2*>(row + NRAND + 4) = make_uint2(0u, 0u);
+    } else if (c <= NRAND + 6) {
+      // columns 16 .. 63, eight at a time
+      *reinterpret_cast<uint4*>(row + 8 * (c - NRAND + 1)) = make_uint4(0u, 0u, 0u, 0u);
+    }
   }
 }
 
@@ -194,11 +242,28 @@ __global__ void agg_bf16_kernel(int n, const int* rp, const int* col, const floa
   for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
        i += (gridDim.x * blockDim.x) >> 5) {
     float a0 = 0.f, a1 = 0.f;
-    for (int q = rp[i]; q < rp[i + 1]; ++q) {
-      const __nv_bfloat162 h = reinterpret_cast<const __nv_bfloat162*>(cat + (size_t)col[q] * CATW)[lane];
-      const float w = val[q];
-      a0 = fmaf(w, __bfloat162float(h.x), a0);
-      a1 = fmaf(w, __bfloat162float(h.y), a1);
+    const int q1 = rp[i + 1];
+    for (int q0 = rp[i]; q0 < q1; q0 += 32) {
+      // the next edges' columns and weights in one load, then their rows four at a time
+      const int cnt = min(32, q1 - q0);
+      const int cl = lane < cnt ? col[q0 + lane] : i;
+      const float wl = lane < cnt ? val[q0 + lane] : 0.f;
+      for (int t = 0; t < cnt; t += 4) {
+        __nv_bfloat162 h[4];
+        float w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int c = __shfl_sync(0xffffffffu, cl, t + u);
+          w[u] = __shfl_sync(0xffffffffu, wl, t + u);
+          h[u] = reinterpret_cast<const __nv_bfloat162*>(cat + (size_t)c * CATW)[lane];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (t + u < cnt) {
+            a0 = fmaf(w[u], __bfloat162float(h[u].x), a0);
+            a1 = fmaf(w[u], __bfloat162float(h[u].y), a1);
+          }
+      }
     }
     reinterpret_cast<__nv_bfloat162*>(cat + (size_t)i * CATW + HID)[lane] = __floats2bfloat162_rn(a0, a1);
   }
@@ -210,27 +275,66 @@ __global__ void agg_back_kernel(int n, const int* rp, const int* col, const floa
   const int lane = threadIdx.x & 31;
   for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
        i += (gridDim.x * blockDim.x) >> 5) {
-    float a0 = dcat[(size_t)i * CATW + 2 * lane], a1 = dcat[(size_t)i * CATW + 2 * lane + 1];
-    for (int q = rp[i]; q < rp[i + 1]; ++q) {
-      const float* src = dcat + (size_t)col[q] * CATW + HID;
-      a0 = fmaf(val[q], src[2 * lane], a0);
-      a1 = fmaf(val[q], src[2 * lane + 1], a1);
+    const float2 own = reinterpret_cast<const float2*>(dcat + (size_t)i * CATW)[lane];
+    float a0 = own.x, a1 = own.y;
+    const int q1 = rp[i + 1];
+    for (int q0 = rp[i]; q0 < q1; q0 += 32) {
+      const int cnt = min(32, q1 - q0);
+      const int cl = lane < cnt ? col[q0 + lane] : i;
+      const float wl = lane < cnt ? val[q0 + lane] : 0.f;
+      for (int t = 0; t < cnt; t += 4) {
+        float2 h[4];
+        float w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int c = __shfl_sync(0xffffffffu, cl, t + u);
+          w[u] = __shfl_sync(0xffffffffu, wl, t + u);
+          h[u] = reinterpret_cast<const float2*>(dcat + (size_t)c * CATW + HID)[lane];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (t + u < cnt) {
+            a0 = fmaf(w[u], h[u].x, a0);
+            a1 = fmaf(w[u], h[u].y, a1);
+          }
+      }
     }
-    dh[(size_t)i * HID + 2 * lane] = a0;
-    dh[(size_t)i * HID + 2 * lane + 1] = a1;
+    reinterpret_cast<float2*>(dh + (size_t)i * HID)[lane] = make_float2(a0, a1);
   }
 }
 
-// ---- heads: U = Z[:, :r] / ||Z[:, :r]||, y = Zy[:, 16] ----
-__global__ void normalize_kernel(int n, int r, const float* zy, float* U, float* nz, float* y) {
+// ---- heads: U = Z[:, :r] / ||Z[:, :r]||, y = Zy[:, 16]; with Ud, yd also the caller's FP64 copies
+// (U n x r without padding) ----
+__global__ void normalize_kernel(int n, int r, const float* zy, float* U, float* nz, float* y,
+                                 double* Ud, double* yd) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const float* z = zy + (size_t)i * HEADW;
+    const float4* zr = reinterpret_cast<const float4*>(zy + (size_t)i * HEADW);
+    float z[RMAX];
+#pragma unroll
+    for (int c = 0; c < RMAX; c += 4) {
+      const float4 x = zr[c / 4];
+      z[c] = x.x; z[c + 1] = x.y; z[c + 2] = x.z; z[c + 3] = x.w;
+    }
+    const float yi = zy[(size_t)i * HEADW + RMAX];
     float s = 0.f;
-    for (int c = 0; c < r; ++c) s = fmaf(z[c], z[c], s);
+#pragma unroll
+    for (int c = 0; c < RMAX; ++c)
+      if (c < r) s = fmaf(z[c], z[c], s);
     const float nrm = sqrtf(fmaxf(s, 1e-30f));
-    for (int c = 0; c < RMAX; ++c) U[(size_t)i * RMAX + c] = c < r ? z[c] / nrm : 0.f;
+#pragma unroll
+    for (int c = 0; c < RMAX; ++c) z[c] = c < r ? z[c] / nrm : 0.f;
+    float4* ur = reinterpret_cast<float4*>(U + (size_t)i * RMAX);
+#pragma unroll
+    for (int c = 0; c < RMAX; c += 4)
+      ur[c / 4] = make_float4(z[c], z[c + 1], z[c + 2], z[c + 3]);
     nz[i] = nrm;
-    y[i] = z[RMAX];
+    y[i] = yi;
+    if (Ud != nullptr) {
+#pragma unroll
+      for (int c = 0; c < RMAX; ++c)
+        if (c < r) Ud[(size_t)i * r + c] = (double)z[c];
+      yd[i] = (double)yi;
+    }
   }
 }
 
@@ -242,31 +346,49 @@ __global__ void loss_grad_kernel(int n, int r, int nedges, const int* rp, const 
   double lsum = 0.0;
   const float invE = 1.f / (float)nedges, invn = 1.f / (float)n;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    // rows of U hold zeros from column r on, so every loop runs over all RMAX columns (in
+    // registers; a loop to r would index them through memory)
     float ui[RMAX], du[RMAX];
-    for (int c = 0; c < RMAX; ++c) {
-      ui[c] = U[(size_t)i * RMAX + c];
-      du[c] = 0.f;
+#pragma unroll
+    for (int c = 0; c < RMAX; c += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(U + (size_t)i * RMAX + c);
+      ui[c] = x.x; ui[c + 1] = x.y; ui[c + 2] = x.z; ui[c + 3] = x.w;
+      du[c] = du[c + 1] = du[c + 2] = du[c + 3] = 0.f;
     }
     for (int q = rp[i]; q < rp[i + 1]; ++q) {
       const int j = col[q];
+      float uj[RMAX];
+#pragma unroll
+      for (int c = 0; c < RMAX; c += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(U + (size_t)j * RMAX + c);
+        uj[c] = x.x; uj[c + 1] = x.y; uj[c + 2] = x.z; uj[c + 3] = x.w;
+      }
       float d = 0.f;
-      for (int c = 0; c < r; ++c) d = fmaf(ui[c], U[(size_t)j * RMAX + c], d);
+#pragma unroll
+      for (int c = 0; c < RMAX; ++c) d = fmaf(ui[c], uj[c], d);
       const float g = d - Xs[eid[q]];
       if (i < j) lsum += (double)g * g * invE;
       const float co = 2.f * g * invE;
-      for (int c = 0; c < r; ++c) du[c] = fmaf(co, U[(size_t)j * RMAX + c], du[c]);
+#pragma unroll
+      for (int c = 0; c < RMAX; ++c) du[c] = fmaf(co, uj[c], du[c]);
     }
     const float ry = y[i] - ys[i];
     lsum += (double)BETA * ry * ry * invn;
     float ud = 0.f;
-    for (int c = 0; c < r; ++c) ud = fmaf(ui[c], du[c], ud);
-    bf16* dh = dhead + (size_t)i * HID;
+#pragma unroll
+    for (int c = 0; c < RMAX; ++c) ud = fmaf(ui[c], du[c], ud);
+    const float nzi = nz[i];
+    __align__(16) bf16 dh[HID];
+#pragma unroll
     for (int c = 0; c < HID; ++c) {
       float v = 0.f;
-      if (c < r) v = (du[c] - ui[c] * ud) / nz[i];
+      if (c < RMAX) v = c < r ? (du[c] - ui[c] * ud) / nzi : 0.f;
       else if (c == RMAX) v = 2.f * BETA * ry * invn;
       dh[c] = __float2bfloat16(v);
     }
+    uint4* out = reinterpret_cast<uint4*>(dhead + (size_t)i * HID);
+#pragma unroll
+    for (int c = 0; c < HID / 8; ++c) out[c] = reinterpret_cast<const uint4*>(dh)[c];
   }
   double v[1] = {lsum};
   block_reduce(v, 1, red);
@@ -275,29 +397,38 @@ __global__ void loss_grad_kernel(int n, int r, int nedges, const int* rp, const 
 
 // ---- dS = dH * (S > 0) -> BF16 ----
 __global__ void relu_back_kernel(int n, const float* dh, const float* S, bf16* ds) {
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)n * HID;
-       t += (size_t)gridDim.x * blockDim.x)
-    ds[t] = __float2bfloat16(S[t] > 0.f ? dh[t] : 0.f);
-}
-
-// ---- deterministic sums: weight-gradient partials over tiles, bias gradients over nodes ----
-__global__ void wgrad_sum_kernel(int tiles, int N, int mrows, const float* partial, float* out,
-                                 int transpose_out) {
-  // out[m][c] (or out[c][m]) = sum_t partial[t][m][c], m < mrows, c < N
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < mrows * N; idx += gridDim.x * blockDim.x) {
-    const int m = idx / N, c = idx % N;
-    double s = 0.0;
-    for (int t = 0; t < tiles; ++t) s += partial[((size_t)t * 128 + m) * N + c];
-    if (transpose_out) out[(size_t)c * mrows + m] = (float)s;
-    else out[(size_t)m * N + c] = (float)s;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)n * HID / 4;
+       t += (size_t)gridDim.x * blockDim.x) {
+    const float4 d = reinterpret_cast<const float4*>(dh)[t];
+    const float4 x = reinterpret_cast<const float4*>(S)[t];
+    reinterpret_cast<__nv_bfloat162*>(ds)[2 * t] =
+        __floats2bfloat162_rn(x.x > 0.f ? d.x : 0.f, x.y > 0.f ? d.y : 0.f);
+    reinterpret_cast<__nv_bfloat162*>(ds)[2 * t + 1] =
+        __floats2bfloat162_rn(x.z > 0.f ? d.z : 0.f, x.w > 0.f ? d.w : 0.f);
   }
 }
 
-__global__ void colsum_bf16_kernel(int n, int cols, const bf16* x, int ldx, float* out) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += gridDim.x * blockDim.x) {
+// ---- deterministic sums over tiles, FP64: the weight gradients' partials (m < mrows, c < N) and
+// the bias gradients' (entry mrows * N + c).  head: the heads' layout of the parameter vector
+// (theta_u, theta_y, b_y), else out is theta (mrows x N) followed by b (N) ----
+__global__ void wgrad_sum_kernel(int tiles, int N, int mrows, const float* partial,
+                                 const double* bias_partial, float* out, int head) {
+  const int nw = mrows * N;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < nw + N; idx += gridDim.x * blockDim.x) {
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s += (double)__bfloat162float(x[(size_t)i * ldx + c]);
-    out[c] = (float)s;
+    if (idx < nw) {
+      const int m = idx / N, c = idx % N;
+      const float* p = partial + (size_t)m * N + c;
+      for (int t = 0; t < tiles; ++t) s += p[(size_t)t * 128 * N];
+      if (!head) out[idx] = (float)s;
+      else if (c < RMAX) out[OFF_THU + m * RMAX + c] = (float)s;
+      else if (c == RMAX) out[OFF_THY + m] = (float)s;
+    } else {
+      const int c = idx - nw;
+      if (head && c != RMAX) continue;
+      for (int t = 0; t < tiles; ++t) s += bias_partial[(size_t)t * N + c];
+      out[head ? OFF_BY : idx] = (float)s;
+    }
   }
 }
 
@@ -416,7 +547,7 @@ double host_normal(uint64_t key, uint64_t e) {
   return std::sqrt(-2.0 * std::log(u1)) * std::cos(2.0 * M_PI * u2);
 }
 
-int forward_impl(lorads_gnn* g, int r, cudaStream_t s) {
+int forward_impl(lorads_gnn* g, int r, cudaStream_t s, double* Ud = nullptr, double* yd = nullptr) {
   const int n = g->n, tiles = (n + 127) / 128;
   const int blocks = 4 * 152;
   prepare_weights_kernel<<<64, 256, 0, s>>>(g->P, g->Bf, g->Bd, g->Bh, g->Bhd);
@@ -437,18 +568,8 @@ int forward_impl(lorads_gnn* g, int r, cudaStream_t s) {
   h.B = g->Bh; h.ldb = HID; h.b_trans = 0; h.b_rows = HEADW; h.b_cols = HID;
   h.rows = n; h.epi = EPI_HEADS; h.out = g->zy; h.bias = g->P + OFF_BY; h.err = g->err;
   GCU((launch_gemm<HEADW, HID>(h, tiles, s)));
-  normalize_kernel<<<blocks, 256, 0, s>>>(n, r, g->zy, g->U, g->nz, g->y);
+  normalize_kernel<<<blocks, 64, 0, s>>>(n, r, g->zy, g->U, g->nz, g->y, Ud, yd);
   return cuda_status(cudaGetLastError());
-}
-
-// head gradients: theta_u[k][c] = gh[k][c] (c < RMAX), theta_y[k] = gh[k][RMAX], b_y = sum dy
-__global__ void scatter_head_grads_kernel(const float* gh, const float* dysum, float* G) {
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < HID * HEADW; idx += gridDim.x * blockDim.x) {
-    const int k = idx / HEADW, c = idx % HEADW;
-    if (c < RMAX) G[OFF_THU + k * RMAX + c] = gh[idx];
-    else if (c == RMAX) G[OFF_THY + k] = gh[idx];
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) G[OFF_BY] = dysum[0];
 }
 
 int backward_impl(lorads_gnn* g, int r, cudaStream_t s) {
@@ -457,17 +578,16 @@ int backward_impl(lorads_gnn* g, int r, cudaStream_t s) {
   loss_grad_kernel<<<152, 256, 0, s>>>(n, r, g->nedges, g->rp, g->col, g->eid, g->U, g->nz,
                                        g->y, g->Xs, g->ys, g->dhead, g->lpart);
   GCU(cudaGetLastError());
-  GCU(cudaMemsetAsync(g->G, 0, sizeof(float) * NPARAM, s));
+  // the bias sums' partials (tiles x 64 doubles) lie in dh, whose contents are used up by then
+  double* const bp = reinterpret_cast<double*>(g->dh);
   // heads: weight gradient H_3^T dhead (64 x 32) and dH_3 = dhead Bhd^T
   {
     GemmArgs w{};
     w.A = g->cat + (size_t)NLAYER * n * CATW; w.lda = CATW; w.a_trans = 1; w.a_cols = HID;
     w.B = g->dhead; w.ldb = HID; w.b_trans = 1; w.b_rows = HEADW; w.b_cols = 0;
-    w.rows = n; w.epi = EPI_WGRAD; w.partial = g->partial; w.err = g->err;
+    w.rows = n; w.epi = EPI_WGRAD; w.partial = g->partial; w.bias_partial = bp; w.err = g->err;
     GCU((launch_gemm<HEADW, 128>(w, tiles, s)));
-    wgrad_sum_kernel<<<8, 256, 0, s>>>(tiles, HEADW, HID, g->partial, g->dcat, 0);
-    colsum_bf16_kernel<<<1, 32, 0, s>>>(n, 1, g->dhead + RMAX, HID, g->dcat + HID * HEADW);
-    scatter_head_grads_kernel<<<8, 256, 0, s>>>(g->dcat, g->dcat + HID * HEADW, g->G);
+    wgrad_sum_kernel<<<33, 64, 0, s>>>(tiles, HEADW, HID, g->partial, bp, g->G, 1);
     GemmArgs d{};
     d.A = g->dhead; d.lda = HID; d.a_trans = 0; d.a_cols = HID;
     d.B = g->Bhd; d.ldb = HID; d.b_trans = 0; d.b_rows = HID; d.b_cols = HID;
@@ -479,10 +599,9 @@ int backward_impl(lorads_gnn* g, int r, cudaStream_t s) {
     GemmArgs w{};
     w.A = g->cat + (size_t)l * n * CATW; w.lda = CATW; w.a_trans = 1; w.a_cols = CATW;
     w.B = g->ds; w.ldb = HID; w.b_trans = 1; w.b_rows = HID; w.b_cols = 0;
-    w.rows = n; w.epi = EPI_WGRAD; w.partial = g->partial; w.err = g->err;
+    w.rows = n; w.epi = EPI_WGRAD; w.partial = g->partial; w.bias_partial = bp; w.err = g->err;
     GCU((launch_gemm<HID, 128>(w, tiles, s)));
-    wgrad_sum_kernel<<<32, 256, 0, s>>>(tiles, HID, CATW, g->partial, g->G + l * LAYER_PARAMS, 0);
-    colsum_bf16_kernel<<<1, 64, 0, s>>>(n, HID, g->ds, HID, g->G + l * LAYER_PARAMS + CATW * HID);
+    wgrad_sum_kernel<<<129, 64, 0, s>>>(tiles, HID, CATW, g->partial, bp, g->G + l * LAYER_PARAMS, 0);
     if (l > 0) {
       GemmArgs d{};
       d.A = g->ds; d.lda = HID; d.a_trans = 0; d.a_cols = HID;
@@ -605,7 +724,8 @@ int lorads_gnn_load_graph(lorads_gnn* g, int64_t n, int64_t nedges, const int32_
       (st = galloc(g, &g->S, (size_t)NLAYER * n * HID)) || (st = galloc(g, &g->zy, (size_t)n * HEADW)) ||
       (st = galloc(g, &g->U, (size_t)n * RMAX)) || (st = galloc(g, &g->nz, n)) ||
       (st = galloc(g, &g->y, n)) || (st = galloc(g, &g->Xs, nedges + 1)) || (st = galloc(g, &g->ys, n)) ||
-      (st = galloc(g, &g->dhead, (size_t)n * HID)) || (st = galloc(g, &g->dh, (size_t)n * HID)) ||
+      (st = galloc(g, &g->dhead, (size_t)n * HID)) ||
+      (st = galloc(g, &g->dh, (size_t)std::max<int64_t>(n, 2) * HID)) ||
       (st = galloc(g, &g->dcat, (size_t)n * CATW + HID * HEADW + 64)) ||
       (st = galloc(g, &g->ds, (size_t)n * HID)) || (st = galloc(g, &g->partial, tiles * 128 * CATW)) ||
       (st = galloc(g, &g->lpart, 152)))
@@ -626,22 +746,18 @@ int lorads_gnn_forward(lorads_gnn* g, int32_t r, double* U0, double* y0, void* s
   if (!g || g->n <= 0 || r < 1 || r > RMAX) return LORADS_ERR_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   GCU(cudaMemsetAsync(g->err, 0, 16, s));
-  int st = forward_impl(g, r, s);
-  if (st != LORADS_OK) return st;
+  // the caller's FP64 outputs are formed on the device (dcat is scratch here) and copied as they are
   const int n = g->n;
-  std::vector<float> hU((size_t)n * RMAX), hy(n);
+  double* const Ud = reinterpret_cast<double*>(g->dcat);
+  double* const yd = Ud + (size_t)n * r;
+  int st = forward_impl(g, r, s, Ud, yd);
+  if (st != LORADS_OK) return st;
   int herr = 0;
-  GCU(cudaMemcpyAsync(hU.data(), g->U, sizeof(float) * n * RMAX, cudaMemcpyDeviceToHost, s));
-  GCU(cudaMemcpyAsync(hy.data(), g->y, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
+  if (U0) GCU(cudaMemcpyAsync(U0, Ud, sizeof(double) * n * r, cudaMemcpyDeviceToHost, s));
+  if (y0) GCU(cudaMemcpyAsync(y0, yd, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
   GCU(cudaMemcpyAsync(&herr, g->err, 4, cudaMemcpyDeviceToHost, s));
   GCU(cudaStreamSynchronize(s));
-  if (herr) return LORADS_ERR_DEVICE;
-  if (U0)
-    for (int i = 0; i < n; ++i)
-      for (int c = 0; c < r; ++c) U0[(size_t)i * r + c] = hU[(size_t)i * RMAX + c];
-  if (y0)
-    for (int i = 0; i < n; ++i) y0[i] = hy[i];
-  return LORADS_OK;
+  return herr ? LORADS_ERR_DEVICE : LORADS_OK;
 }
 
 int lorads_gnn_train_step(lorads_gnn* g, int32_t r, const double* Xs, const double* ys, double lr,
