@@ -442,6 +442,7 @@ struct BlockScope {
     return true;
   }
   __device__ bool is_leader() const { return threadIdx.x == 0; }
+  __device__ bool leader_cta() const { return true; }
 };
 
 // a CTA's partial sum of one value and the number of the barrier it belongs to, stored and
@@ -547,6 +548,7 @@ struct GridScope {
   __device__ int tid() const { return ((int)blockIdx.x - first) * blockDim.x + threadIdx.x; }
   __device__ int nthreads() const { return count() * blockDim.x; }
   __device__ bool is_leader() const { return (int)blockIdx.x == first && threadIdx.x == 0; }
+  __device__ bool leader_cta() const { return (int)blockIdx.x == first; }
 
   // clears the failure mark; every thread, once, before the scope's first barrier
   __device__ void init() {

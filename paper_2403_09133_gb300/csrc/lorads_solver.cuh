@@ -731,14 +731,19 @@ struct Solver {
       int it = 0;
       bool stalled = false;
       for (;;) {
-        rp = sqrt(e2) / (1.0 + P.b_inf);
-        const double grel = sqrt(g2) / (1.0 + P.C_fro);
+        const int newest = (head - 1 + ring) % ring;
+        double s4[4];
+        once<3>(s4, [&](double* o) {
+          o[0] = sqrt(e2) / (1.0 + P.b_inf);
+          o[1] = sqrt(g2) / (1.0 + P.C_fro);
+          o[2] = cnt > 0 ? hsy[newest] / hyy[newest] : 1.0;
+        });
+        rp = s4[0];
+        const double grel = s4[1], H0 = s4[2];
         if (!(grel == grel)) { status = ST_NAN; return true; }
         if (grel <= fmax(1e-12, fmin(prm.inner_tol_max, prm.inner_tol_factor * rp))) break;
         if (it >= prm.inner_max_iter) { stalled = true; break; }
         double dg;
-        const int newest = (head - 1 + ring) % ring;
-        const double H0 = cnt > 0 ? hsy[newest] / hyy[newest] : 1.0;
         if (!lbfgs_direction(cnt, head, hrho, H0, dg)) return false;
         if (dg >= 0.0) {
           if (!steepest()) return false;
@@ -747,7 +752,8 @@ struct Solver {
         }
         double a[4];
         if (!line_search_coeffs(sigma, a)) return false;
-        const double t = quartic_step(a[0], a[1], a[2], a[3]);
+        double t;
+        once<1>(&t, [&](double* o) { o[0] = quartic_step(a[0], a[1], a[2], a[3]); });
         if (!(t > 0.0)) {
           if (cnt > 0) { cnt = 0; head = 0; continue; }
           break;
@@ -758,7 +764,7 @@ struct Solver {
         double sy, yy;
         if (!history_pair(head, sy, yy)) return false;
         if (sy > 0.0) {
-          hrho[head] = 1.0 / sy;
+          once<1>(&hrho[head], [&](double* o) { o[0] = 1.0 / sy; });
           hsy[head] = sy;
           hyy[head] = yy;
           head = (head + 1) % ring;
@@ -862,11 +868,20 @@ struct Solver {
     }
     if (!sc.reduce(v, 2)) return false;
     ++hess;
-    double rr = v[0];
-    const double target = fmax(prm.cg_rel_tol * sqrt(rr), prm.cg_abs_floor * sqrt(v[1]));
     const T rho_t = (T)rho, gamma_t = (T)gamma;
     int it = 0;
-    while (sqrt(rr) > target && it < prm.cg_max_iter) {
+    // thread 0 carries r.r and the stopping target in shared memory and evaluates alpha and beta
+    double* const own = sc.scratch() + 12;
+    if (threadIdx.x == 0) {
+      const double rr = v[0];
+      own[0] = rr;
+      own[1] = fmax(prm.cg_rel_tol * sqrt(rr), prm.cg_abs_floor * sqrt(v[1]));
+      cg_leave(sqrt(rr) > own[1] ? 0 : 1, 0.0, 0.0);
+    }
+    __syncthreads();
+    T alpha_t, beta_t;
+    int state = cg_take(alpha_t, beta_t);
+    while (state == 0 && it < prm.cg_max_iter) {
       // HP = H P, p.Hp
       double w[1] = {0.0};
       if (multi && !con_q<T>(A.Pd, Wt)) return false;
@@ -881,15 +896,14 @@ struct Solver {
         const T d = team_sum(frag_dot_local(Pj, Hj), st);
         if (wr.sub == 0 && st.lead) w[0] += (double)d;
       }
-      if (!sc.reduce(w, 1)) return false;
+      if (!sc.reduce_each(w, 1, [this, own](int, double pHp) {
+            if (!(pHp > 0.0)) cg_leave(pHp == pHp ? 1 : 2, 0.0, 0.0);
+            else cg_leave(0, own[0] / pHp, 0.0);
+          }))
+        return false;
       ++hess;
-      const double pHp = w[0];
-      if (!(pHp > 0.0)) {
-        if (!(pHp == pHp)) status = ST_NAN;
-        break;
-      }
-      const double alpha = rr / pHp;
-      const T alpha_t = (T)alpha;
+      state = cg_take(alpha_t, beta_t);
+      if (state != 0) break;
       double z[1] = {0.0};
       for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
         const Team& tm = rows.t;
@@ -908,12 +922,20 @@ struct Solver {
         const double d = frag_dot(Rd, Rd, tm);
         if (tm.lead) z[0] += d;
       }
-      if (!sc.reduce(z, 1)) return false;
+      if (!sc.reduce_each(z, 1, [this, own](int, double rr_new) {
+            // stop on the new residual; beta otherwise (a NaN goes on, as p.Hp then shows it)
+            if (sqrt(rr_new) <= own[1]) {
+              cg_leave(1, 0.0, 0.0);
+            } else {
+              // go on while ||r|| > target (false for a NaN, which ends the loop)
+              cg_leave(sqrt(rr_new) > own[1] ? 0 : 3, 0.0, rr_new / own[0]);
+              own[0] = rr_new;
+            }
+          }))
+        return false;
       ++it;
-      const double rr_new = z[0];
-      if (sqrt(rr_new) <= target) { rr = rr_new; break; }
-      const T beta_t = (T)(rr_new / rr);
-      rr = rr_new;
+      state = cg_take(alpha_t, beta_t);
+      if (state == 1) break;
       for (TeamRows rows(this->tm, n); rows.more(); rows.next()) {
         const Team& tm = rows.t;
         const int j = rows.j;
@@ -1135,9 +1157,13 @@ struct Solver {
       if (!sc.reduce(v, 5)) return false;
       admm_iters = k + 1;
       log_iter(k, rho, v[0], v[1], v[4]);
-      const double rp = sqrt(v[0]) / (1.0 + P.b_inf);
-      const double rph = sqrt(v[1]) / (1.0 + P.b_inf);
-      const double rs = gamma * sqrt(v[2]) / (1.0 + sqrt(v[3]));
+      double s3[3];
+      once<3>(s3, [&](double* o) {
+        o[0] = sqrt(v[0]) / (1.0 + P.b_inf);
+        o[1] = sqrt(v[1]) / (1.0 + P.b_inf);
+        o[2] = gamma * sqrt(v[2]) / (1.0 + sqrt(v[3]));
+      });
+      const double rp = s3[0], rph = s3[1], rs = s3[2];
       last_rs = rs;
       if (!(rp == rp) || !(rs == rs)) { status = ST_NAN; break; }
       if (rph <= prm.tol) {
@@ -1468,6 +1494,19 @@ struct Solver {
     }
     cg_iters += it;
     return true;
+  }
+
+  // f(out) in thread 0 of every CTA, whose K results every thread receives in v: scalars with FP64
+  // divisions, square roots and the like are evaluated once per CTA (a division in nine warps takes
+  // 1,270 clocks of the SM's FP64 unit, in one warp 430; a square root 1,340 and 675)
+  template <int K, class F>
+  __device__ __forceinline__ void once(double* v, F f) {
+    double* own = sc.scratch() + 24;
+    if (threadIdx.x == 0) f(own);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] = own[i];
+    __syncthreads();
   }
 
   // What thread 0 of a CTA leaves for its threads after a reduction of a CG: the state (0 go on,
@@ -2603,20 +2642,38 @@ struct Solver {
           b2[c] += w * w;
         }
       }
-      if (!sc.reduce(b2, NC)) return false;
+      // beta_k = ||W||, the scale of q_{k+1} and the column's length, for each column in the thread
+      // that holds its sum; every thread reads them from the scratch row
+      double* const nxt = sc.scratch();     // 1/beta, beta, length of the four columns
+      if (!sc.reduce_each(b2, NC, [&](int c, double w2) {
+            double ac = a[0], bc = bp[0];
+            int lc = len[0];
+#pragma unroll
+            for (int q = 1; q < NC; ++q)
+              if (q == c) {
+                ac = a[q];
+                bc = bp[q];
+                lc = len[q];
+              }
+            const double beta = sqrt(w2);
+            if (sc.leader_cta()) {
+              hist[8 * k + c] = ac;
+              hist[8 * k + 4 + c] = beta;
+            }
+            const bool live = lc > k + 1;
+            const bool breakdown = !(beta > 1e-12 * (fabs(ac) + bc) && beta > 1e-300);
+            if (live && breakdown) lc = k + 1;
+            nxt[c] = lc > k + 1 ? 1.0 / beta : 0.0;
+            nxt[NC + c] = lc > k + 1 ? beta : 0.0;
+            nxt[2 * NC + c] = (double)lc;
+          }))
+        return false;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        const double beta = sqrt(b2[c]);
-        if (sc.is_leader()) {
-          hist[8 * k + c] = a[c];
-          hist[8 * k + 4 + c] = beta;
-        }
-        const bool live = len[c] > k + 1;
-        const bool breakdown = !(beta > 1e-12 * (fabs(a[c]) + bp[c]) && beta > 1e-300);
-        if (live && breakdown) len[c] = k + 1;
         qps[c] = qs[c];
-        qs[c] = len[c] > k + 1 ? 1.0 / beta : 0.0;
-        bp[c] = len[c] > k + 1 ? beta : 0.0;
+        qs[c] = nxt[c];
+        bp[c] = nxt[NC + c];
+        len[c] = (int)nxt[2 * NC + c];
       }
       double* t = Qp;
       Qp = Q;
