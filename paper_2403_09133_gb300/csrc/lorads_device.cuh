@@ -835,7 +835,8 @@ __device__ void spmm_row_warp(const DevProblem& P, const T* Wm, int ld, int j, c
   }
   const T* av = aval<T>(P);
   const bool a_part = (wb != 0.0) || (lam != nullptr) || (e != nullptr);
-  if (a_part) {
+  if (a_part && sizeof(T) == 8) {
+    // FP64: the products outweigh the weights, and four rows in flight would halve the warps
     const int q1 = P.A_rp[j + 1];
     int q = P.A_rp[j] + w.sub;
     for (; q + w.S < q1; q += 2 * w.S) {
@@ -858,6 +859,43 @@ __device__ void spmm_row_warp(const DevProblem& P, const T* Wm, int ld, int j, c
       Frag<T> Wk;
       frag_load(Wk, Wm, P.A_col[q], ld, t);
       frag_axpy(acc, (T)(c * (double)av[q]), Wk);
+    }
+  } else if (a_part) {
+    // 32 entries a round: lane l forms the weight of entry l once (FP64, whose instructions take 16
+    // clocks of the SM each whatever the lanes do: with every sub-team forming its own, the
+    // weights of 8 entries cost as much as those of 32 here), then sub-team s takes the entries
+    // s, s + S, ..., their rows all in flight
+    const int lane = threadIdx.x & 31;
+    const int q1 = P.A_rp[j + 1];
+    __syncwarp();
+    for (int q0 = P.A_rp[j]; q0 < q1; q0 += 32) {
+      int col = j;
+      T c = T(0);
+      if (q0 + lane < q1) {
+        const int q = q0 + lane, i = P.A_con[q];
+        col = P.A_col[q];
+        double x = wb * P.b[i];
+        if (lam) x += wl * lam[i];
+        if (e) x += we * e[i];
+        c = (T)(x * (double)av[q]);
+      }
+      const int rounds = min(32, q1 - q0);
+      for (int s0 = 0; s0 < rounds; s0 += 4 * w.S) {
+        Frag<T> Wk[4];
+        T ck[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int src = s0 + u * w.S + w.sub;          // < 32 when it is one of the entries
+          const int k = __shfl_sync(0xffffffffu, col, src & 31);
+          ck[u] = __shfl_sync(0xffffffffu, c, src & 31);
+          Team tw = t;
+          tw.nc = src < rounds ? t.nc : 0;
+          frag_load(Wk[u], Wm, k, ld, tw);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (s0 + u * w.S + w.sub < rounds) frag_axpy(acc, ck[u], Wk[u]);
+      }
     }
   }
   frag_warp_combine(acc, t.G);

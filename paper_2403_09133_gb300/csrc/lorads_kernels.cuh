@@ -102,27 +102,184 @@ __global__ void op_spmm_kernel(DevProblem P, int ld, const double* w, double gam
   }
 }
 
+// Diagonal constraints: a pass over P, V and the result, bound by HBM.  A kernel of its own: with
+// the many-entries form in one kernel it took that form's 72 registers, half the warps.
+template <typename T>
+__global__ void __launch_bounds__(256, 5)
+op_hessian_diag_kernel(DevProblem P, int ld, T rho, T gamma, const T* V, const T* Pm, T* out) {
+  const Team t = make_team(ld, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  const T* ra = rowa<T>(P);
+  for (TeamRows rows(t, P.n); rows.more(); rows.next()) {
+    Frag<T> Pj, Vj, H;
+    frag_load(Pj, Pm, rows.j, ld, rows.t);
+    frag_load(Vj, V, rows.j, ld, rows.t);
+    hessian_row<T>(ra[rows.j], Vj, Pj, rho, gamma, rows.t, H);
+    frag_store(H, out, rows.j, ld, rows.t);
+  }
+}
+
 template <typename T>
 __global__ void op_hessian_kernel(DevProblem P, int ld, T rho, T gamma, const T* V, const T* Pm,
                                   T* out) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-  if (P.a_diag_only) {
-    const Team t = make_team(ld, tid, nt);
-    const T* ra = rowa<T>(P);
-    for (TeamRows rows(t, P.n); rows.more(); rows.next()) {
-      Frag<T> Pj, Vj, H;
-      frag_load(Pj, Pm, rows.j, ld, rows.t);
-      frag_load(Vj, V, rows.j, ld, rows.t);
-      hessian_row<T>(ra[rows.j], Vj, Pj, rho, gamma, rows.t, H);
-      frag_store(H, out, rows.j, ld, rows.t);
+  const WarpRow wr =
+      make_warp_row(ld, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  for (int j = wr.warp; j < P.n; j += wr.nwarps) {
+    Frag<T> Pj, H;
+    frag_load(Pj, Pm, j, ld, wr.st);
+    hessian_row_warp<T>(P, V, Pm, ld, j, Pj, rho, gamma, wr, H);
+    if (wr.sub == 0) frag_store(H, out, j, ld, wr.st);
+  }
+}
+
+// ---- FP64 operators.  FP64 issues one warp instruction per SM every 16 clocks whatever its lanes
+// do (1/64 of the FP32 rate), so these kernels are bound by the FP64 instructions they issue, and
+// the layout keeps those few: a row of ld doubles is ld / 2 units of 16 bytes, dealt to G lanes (lane
+// l: units l, l + G, ...), N units per lane with G the smallest power of two that gives N <= 8.  The
+// solver's layout (4-element chunks, two per lane) leaves a third of the lanes of a ld = 20 row
+// without elements in instructions that are issued all the same.
+struct UnitRow {
+  int G, lane, id, count, units;   // id, count: teams of the grid
+};
+__device__ inline UnitRow make_unit_row(int ld, int G) {
+  UnitRow t;
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+  t.G = G;
+  t.lane = tid & (G - 1);
+  t.id = tid / G;
+  t.count = gridDim.x * blockDim.x / G;
+  t.units = ld / 2;
+  return t;
+}
+__device__ __forceinline__ double2 unit_at(const double* row, int u, int units) {
+  return u < units ? *reinterpret_cast<const double2*>(row + 2 * u) : make_double2(0.0, 0.0);
+}
+__device__ __forceinline__ double team_sum64(double x, int G) {
+  for (int off = G >> 1; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  return x;
+}
+
+// <A_i, U V^T>: one team per constraint
+template <int N>
+__global__ void __launch_bounds__(256) op_sddmm_f64_kernel(DevProblem P, int ld, int G,
+                                                           const double* U, const double* V,
+                                                           double* q) {
+  const UnitRow t = make_unit_row(ld, G);
+  const int sub = (threadIdx.x & 31) / G;
+  for (int i0 = t.id - sub; i0 < P.m; i0 += t.count) {
+    const bool live = i0 + sub < P.m;
+    const int i = live ? i0 + sub : P.m - 1;
+    const int e0 = P.con_ptr[i], cnt = live ? P.con_ptr[i + 1] - e0 : 0;
+    const int rounds = P.a_multi ? __reduce_max_sync(0xffffffffu, cnt) : 1;
+    double s = 0.0;
+    for (int k = 0; k < rounds; ++k) {
+      const int e = k < cnt ? e0 + k : e0;
+      const int r = P.con_r[e], c = P.con_c[e];
+      const double a = P.con_a[e];
+      const double* Ur = U + (size_t)r * ld;
+      const double* Vc = V + (size_t)c * ld;
+      const double* Uc = U + (size_t)c * ld;
+      const double* Vr = V + (size_t)r * ld;
+      double x = 0.0, y = 0.0;
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const double2 p = unit_at(Ur, t.lane + G * u, t.units);
+        const double2 v = unit_at(Vc, t.lane + G * u, t.units);
+        x = fma(p.x, v.x, x);
+        y = fma(p.y, v.y, y);
+      }
+      if (r != c) {
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+          const double2 p = unit_at(Uc, t.lane + G * u, t.units);
+          const double2 v = unit_at(Vr, t.lane + G * u, t.units);
+          x = fma(p.x, v.x, x);
+          y = fma(p.y, v.y, y);
+        }
+      }
+      __syncwarp();
+      x = a * team_sum64(x + y, G);
+      if (k < cnt) s += x;
     }
-  } else {
-    const WarpRow wr = make_warp_row(ld, tid, nt);
-    for (int j = wr.warp; j < P.n; j += wr.nwarps) {
-      Frag<T> Pj, H;
-      frag_load(Pj, Pm, j, ld, wr.st);
-      hessian_row_warp<T>(P, V, Pm, ld, j, Pj, rho, gamma, wr, H);
-      if (wr.sub == 0) frag_store(H, out, j, ld, wr.st);
+    if (live && t.lane == 0) q[i] = s;
+  }
+}
+
+// (A^T(w) - C) V + gamma V with diagonal constraints: one team per row, C's entries two at a time; the
+// row's own terms a w + gamma in one product
+template <int N>
+__global__ void __launch_bounds__(256) op_spmm_f64_diag_kernel(DevProblem P, int ld, int G,
+                                                               const double* w, double gamma,
+                                                               const double* V, double* out) {
+  const UnitRow t = make_unit_row(ld, G);
+  for (int j = t.id; j < P.n; j += t.count) {
+    const int con = P.row_con[j];
+    const double own = con >= 0 ? fma(P.row_a[j], w[con], gamma) : gamma;
+    double2 acc[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) acc[u] = make_double2(0.0, 0.0);
+    int q = P.C_rp[j];
+    const int q1 = P.C_rp[j + 1];
+    for (; q + 2 <= q1; q += 2) {
+      const double* V0 = V + (size_t)P.C_col[q] * ld;
+      const double* V1 = V + (size_t)P.C_col[q + 1] * ld;
+      const double c0 = -P.C_val[q], c1 = -P.C_val[q + 1];
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const double2 x = unit_at(V0, t.lane + G * u, t.units);
+        const double2 y = unit_at(V1, t.lane + G * u, t.units);
+        acc[u].x = fma(c1, y.x, fma(c0, x.x, acc[u].x));
+        acc[u].y = fma(c1, y.y, fma(c0, x.y, acc[u].y));
+      }
+    }
+    if (q < q1) {
+      const double* V0 = V + (size_t)P.C_col[q] * ld;
+      const double c0 = -P.C_val[q];
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const double2 x = unit_at(V0, t.lane + G * u, t.units);
+        acc[u].x = fma(c0, x.x, acc[u].x);
+        acc[u].y = fma(c0, x.y, acc[u].y);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u)
+      if (t.lane + G * u < t.units) {
+        const double2 x = unit_at(V + (size_t)j * ld, t.lane + G * u, t.units);
+        *reinterpret_cast<double2*>(out + (size_t)j * ld + 2 * (t.lane + G * u)) =
+            make_double2(fma(own, x.x, acc[u].x), fma(own, x.y, acc[u].y));
+      }
+  }
+}
+
+// eq. linU's matrix with diagonal constraints: gamma P_j + rho a^2 (P_j . V_j) V_j, one team per row
+template <int N>
+__global__ void __launch_bounds__(256) op_hessian_f64_diag_kernel(DevProblem P, int ld, int G,
+                                                                  double rho, double gamma,
+                                                                  const double* V,
+                                                                  const double* Pm, double* out) {
+  const UnitRow t = make_unit_row(ld, G);
+  const int sub = (threadIdx.x & 31) / G;
+  for (int j0 = t.id - sub; j0 < P.n; j0 += t.count) {
+    const bool live = j0 + sub < P.n;
+    const int j = live ? j0 + sub : P.n - 1;
+    const double a = P.row_a[j];
+    double2 p[N], v[N];
+    double x = 0.0, y = 0.0;
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      p[u] = unit_at(Pm + (size_t)j * ld, t.lane + G * u, t.units);
+      v[u] = unit_at(V + (size_t)j * ld, t.lane + G * u, t.units);
+      x = fma(p[u].x, v[u].x, x);
+      y = fma(p[u].y, v[u].y, y);
+    }
+    __syncwarp();
+    const double c = rho * (a * (a * team_sum64(x + y, G)));
+    if (live) {
+#pragma unroll
+      for (int u = 0; u < N; ++u)
+        if (t.lane + G * u < t.units)
+          *reinterpret_cast<double2*>(out + (size_t)j * ld + 2 * (t.lane + G * u)) =
+              make_double2(fma(c, v[u].x, gamma * p[u].x), fma(c, v[u].y, gamma * p[u].y));
     }
   }
 }
@@ -278,16 +435,63 @@ struct Launch {
 LORADS_DECLARE_LAUNCH(double)
 LORADS_DECLARE_LAUNCH(float)
 
+// lanes per row and units per lane of the FP64 operators (ld <= 256: at most 16 lanes)
+inline int unit_lanes(int ld) {
+  int G = 1;
+  while ((ld / 2 + G - 1) / G > 8) G <<= 1;
+  return G < 2 ? 2 : G;
+}
+template <template <int> class K, class... A>
+inline cudaError_t launch_units(int ld, A... args) {
+  const int G = unit_lanes(ld);
+  switch ((ld / 2 + G - 1) / G) {
+    case 1: K<1>::go(G, args...); break;
+    case 2: K<2>::go(G, args...); break;
+    case 3: K<3>::go(G, args...); break;
+    case 4: K<4>::go(G, args...); break;
+    case 5: K<5>::go(G, args...); break;
+    case 6: K<6>::go(G, args...); break;
+    case 7: K<7>::go(G, args...); break;
+    default: K<8>::go(G, args...); break;
+  }
+  return cudaGetLastError();
+}
+template <int N>
+struct SddmmF64 {
+  static void go(int G, int grid, cudaStream_t s, const DevProblem& P, int ld, const double* U,
+                 const double* V, double* q) {
+    op_sddmm_f64_kernel<N><<<grid, 256, 0, s>>>(P, ld, G, U, V, q);
+  }
+};
+template <int N>
+struct SpmmF64Diag {
+  static void go(int G, int grid, cudaStream_t s, const DevProblem& P, int ld, const double* w,
+                 double gamma, const double* V, double* out) {
+    op_spmm_f64_diag_kernel<N><<<grid, 256, 0, s>>>(P, ld, G, w, gamma, V, out);
+  }
+};
+template <int N>
+struct HessianF64Diag {
+  static void go(int G, int grid, cudaStream_t s, const DevProblem& P, int ld, double rho,
+                 double gamma, const double* V, const double* Pm, double* out) {
+    op_hessian_f64_diag_kernel<N><<<grid, 256, 0, s>>>(P, ld, G, rho, gamma, V, Pm, out);
+  }
+};
+
 #define LORADS_DEFINE_LAUNCH(T)                                                                \
   template <>                                                                                  \
   cudaError_t Launch<T>::op_sddmm(const DevProblem& P, int ld, const T* U, const T* V,         \
                                   double* q, int grid, cudaStream_t s) {                       \
-    op_sddmm_kernel<T><<<grid, 256, 0, s>>>(P, ld, U, V, q);                                   \
+    if constexpr (sizeof(T) == 8) return launch_units<SddmmF64>(ld, grid, s, P, ld, U, V, q);  \
+    else op_sddmm_kernel<T><<<grid, 256, 0, s>>>(P, ld, U, V, q);                              \
     return cudaGetLastError();                                                                 \
   }                                                                                            \
   template <>                                                                                  \
   cudaError_t Launch<T>::op_spmm(const DevProblem& P, int ld, const double* w, double gamma,   \
                                  const T* V, T* out, int grid, cudaStream_t s) {               \
+    if constexpr (sizeof(T) == 8) {                                                            \
+      if (P.a_diag_only) return launch_units<SpmmF64Diag>(ld, grid, s, P, ld, w, gamma, V, out); \
+    }                                                                                          \
     op_spmm_kernel<T><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);                           \
     return cudaGetLastError();                                                                 \
   }                                                                                            \
@@ -296,10 +500,15 @@ LORADS_DECLARE_LAUNCH(float)
                                     const T* V, const T* Pm, T* out, int grid,                 \
                                     cudaStream_t s) {                                          \
     if (P.a_multi) {                                                                           \
-      op_sddmm_kernel<T><<<grid, 256, 0, s>>>(P, ld, Pm, V, P.op_q);                           \
+      const cudaError_t e = op_sddmm(P, ld, Pm, V, P.op_q, grid, s);                           \
+      if (e != cudaSuccess) return e;                                                          \
       op_hessian_q_kernel<T><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, P.op_q, out); \
-    } else {                                                                                   \
+    } else if (!P.a_diag_only) {                                                               \
       op_hessian_kernel<T><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, out);          \
+    } else if constexpr (sizeof(T) == 8) {                                                     \
+      return launch_units<HessianF64Diag>(ld, grid, s, P, ld, rho, gamma, V, Pm, out);         \
+    } else {                                                                                   \
+      op_hessian_diag_kernel<T><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, out);     \
     }                                                                                          \
     return cudaGetLastError();                                                                 \
   }
