@@ -25,6 +25,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lorads_convert.h"
+
 namespace lorads {
 
 constexpr int KMAX = 2;      // chunks per lane
@@ -211,13 +213,20 @@ __device__ __forceinline__ void frag_store(const Frag<T>& f, T* base, long long 
   }
 }
 
+// conversions between element types off the FP64 unit (lorads_convert.h; the same values)
+__device__ __forceinline__ double to_double(float x) { return widen(x); }
+__device__ __forceinline__ double to_double(double x) { return x; }
+template <typename D> __device__ __forceinline__ D from_double(double x);
+template <> __device__ __forceinline__ float from_double<float>(double x) { return narrow(x); }
+template <> __device__ __forceinline__ double from_double<double>(double x) { return x; }
+
 // convert between element types (FP64 master <-> FP32 shadow)
 template <typename D, typename S>
 __device__ __forceinline__ void frag_convert(Frag<D>& d, const Frag<S>& s) {
 #pragma unroll
   for (int k = 0; k < KMAX; ++k)
 #pragma unroll
-    for (int e = 0; e < CHUNK; ++e) d.v[k][e] = D(s.v[k][e]);
+    for (int e = 0; e < CHUNK; ++e) d.v[k][e] = from_double<D>(to_double(s.v[k][e]));
 }
 
 // lane-local partial dot product, accumulated in T
@@ -716,7 +725,7 @@ __device__ __forceinline__ double sddmm_entry(const T* Um, const T* Vm, int ld, 
     frag_load(Vr, Vm, r, ld, t);
     loc += frag_dot_local(Uc, Vr);
   }
-  return a * (double)team_sum(loc, t);
+  return a * to_double(team_sum(loc, t));
 }
 
 // <A_i, U V^T>: the sum over constraint i's entries (team-cooperative; called by whole warps, whose
@@ -877,7 +886,7 @@ __device__ void spmm_row_warp(const DevProblem& P, const T* Wm, int ld, int j, c
         double x = wb * P.b[i];
         if (lam) x += wl * lam[i];
         if (e) x += we * e[i];
-        c = (T)(x * (double)av[q]);
+        c = from_double<T>(x * to_double(av[q]));
       }
       const int rounds = min(32, q1 - q0);
       for (int s0 = 0; s0 < rounds; s0 += 4 * w.S) {

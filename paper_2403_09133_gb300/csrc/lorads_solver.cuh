@@ -555,8 +555,8 @@ struct Solver {
       spmm_row<E>(P, Ub, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, E(0), tm, mCU);
       spmm_row<E>(P, Dt, ld, j, nullptr, nullptr, 0.0, 0.0, 0.0, E(0), tm, mCD);
       frag_load(Dj, Dt, j, ld, tm);
-      const double c1 = -2.0 * (double)frag_dot(Dj, mCU, tm);
-      const double c2 = -(double)frag_dot(Dj, mCD, tm);
+      const double c1 = -2.0 * to_double(frag_dot(Dj, mCU, tm));
+      const double c2 = -to_double(frag_dot(Dj, mCD, tm));
       if (tm.lead) {
         v[7] += c1;
         v[8] += c2;
@@ -593,8 +593,8 @@ struct Solver {
         frag_load(Uc, Ub, cc, ld, tmc);
         E loc = frag_dot_local(Ur, Dc);
         if (rr != cc) loc += frag_dot_local(Uc, Dr);
-        const double e1 = 2.0 * aa * (double)team_sum(loc, tmc);
-        const double e2 = (rr != cc ? 2.0 : 1.0) * aa * (double)frag_dot(Dr, Dc, tmc);
+        const double e1 = 2.0 * aa * to_double(team_sum(loc, tmc));
+        const double e2 = (rr != cc ? 2.0 : 1.0) * aa * to_double(frag_dot(Dr, Dc, tmc));
         if (tmc.lead) accumulate(i, e1, e2);
       }
     }
@@ -894,7 +894,7 @@ struct Solver {
           hessian_row_warp<T>(P, Wt, A.Pd, ld, j, Pj, rho_t, gamma_t, wr, Hj);
         if (wr.sub == 0) frag_store(Hj, A.HP, j, ld, st);
         const T d = team_sum(frag_dot_local(Pj, Hj), st);
-        if (wr.sub == 0 && st.lead) w[0] += (double)d;
+        if (wr.sub == 0 && st.lead) w[0] += to_double(d);
       }
       if (!sc.reduce_each(w, 1, [this, own](int, double pHp) {
             if (!(pHp > 0.0)) cg_leave(pHp == pHp ? 1 : 2, 0.0, 0.0);
@@ -1252,8 +1252,8 @@ struct Solver {
     frag_store(wt, A.HP, j, ld, tm);
     gt = rt;
     frag_axpy(gt, (T)cg, Wjt);
-    const double d1 = (double)frag_dot(rt, rt, tm), d2 = (double)frag_dot(wt, rt, tm);
-    const double d3 = (double)frag_dot(gt, gt, tm);
+    const double d1 = to_double(frag_dot(rt, rt, tm)), d2 = to_double(frag_dot(wt, rt, tm));
+    const double d3 = to_double(frag_dot(gt, gt, tm));
     if (tm.lead) {
       g3[0] += d1;
       g3[1] += d2;
@@ -1347,10 +1347,10 @@ struct Solver {
                                            double& z1) const {
     if (!tm.live) return;
     if (tm.G >= 2) {
-      z0 += (double)((tm.lane & 1) ? d2 : d1);
+      z0 += to_double((tm.lane & 1) ? d2 : d1);
     } else {
-      z0 += (double)d1;
-      z1 += (double)d2;
+      z0 += to_double(d1);
+      z1 += to_double(d2);
     }
   }
   // p = r + b p, s = H p, x += a p, r -= a s, w = H r; stores p, x, r; z += (r.r, w.r)
@@ -1601,7 +1601,7 @@ struct Solver {
         frag_axpy(Xt, T(1), x);                   // shadow of V^{k+1} = shadow(U^{k+1}) + delta
         frag_axpy(dV, T(-1), Vot);
         frag_axpy(dV, T(1), x);
-        const double d2 = (double)frag_dot(dV, dV, tm), o2 = (double)frag_dot(Vot, Vot, tm);
+        const double d2 = to_double(frag_dot(dV, dV, tm)), o2 = to_double(frag_dot(Vot, Vot, tm));
         if (exact) frag_convert(Xt, Xj);          // re-rounded from the master every 32
         // dual step lambda_i += rho (a U_j.V_j - b_i)
         double e = 0.0, lam_new = 0.0;
@@ -1735,7 +1735,7 @@ struct Solver {
         frag_axpy(Xt, T(1), x);                   // shadow of V^{k+1} = shadow(U^{k+1}) + delta
         frag_axpy(dVk, T(-1), Vot);
         frag_axpy(dVk, T(1), x);
-        const double d2 = (double)frag_dot(dVk, dVk, tm), o2 = (double)frag_dot(Vot, Vot, tm);
+        const double d2 = to_double(frag_dot(dVk, dVk, tm)), o2 = to_double(frag_dot(Vot, Vot, tm));
         if (exact) frag_convert(Xt, Xj);          // re-rounded from the master every 32
         // dual step lambda_i += rho (a U_j.V_j - b_i)
         double e = 0.0, lam_new = 0.0;
@@ -1988,7 +1988,7 @@ struct Solver {
       const T u2 = frag_dot(Uj, Uj, tm);
       sphere_hess_row(j, Rb[0], r, Uj, u2, (T)A.e[j], tm, w);
       frag_store(w, Wb[0], j, ld, tm);
-      const double d1 = (double)frag_dot(r, r, tm), d2 = (double)frag_dot(w, r, tm);
+      const double d1 = to_double(frag_dot(r, r, tm)), d2 = to_double(frag_dot(w, r, tm));
       if (tm.lead) {
         g3[0] += d1;
         g3[1] += d2;
@@ -2140,7 +2140,7 @@ struct Solver {
       sphere_hess_row(j, A.Dl, dj, Uj, u2, (T)A.e[j], tm, w);
       frag_load(gj, A.grad, j, ld, tm);
       frag_convert(dd, dj);
-      const double a1 = frag_dot(gj, dd, tm), a2 = (double)frag_dot(dj, w, tm);
+      const double a1 = frag_dot(gj, dd, tm), a2 = to_double(frag_dot(dj, w, tm));
       if (tm.lead) {
         v[0] += a1;
         v[1] += a2;
