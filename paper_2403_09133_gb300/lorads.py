@@ -160,12 +160,11 @@ def _host(a, dtype):
 
 
 def _dev(x):
-    """Device pointer of a torch CUDA tensor, or an integer address, or None."""
-    if x is None:
-        return None
-    if isinstance(x, int):
-        return ctypes.c_void_p(x)
-    return ctypes.c_void_p(x.data_ptr())
+    """Device pointer of a torch CUDA tensor, or an integer address, or None (a plain integer: the
+    argument types make a pointer of it, without an object of its own per argument)."""
+    if x is None or isinstance(x, int):
+        return x
+    return x.data_ptr()
 
 
 def _check(code: int, what: str) -> int:
@@ -318,9 +317,9 @@ class TorchAllocator:
 
 
 def _stream_ptr(stream):
-    if stream is None:
-        return None
-    return ctypes.c_void_p(stream if isinstance(stream, int) else stream.cuda_stream)
+    if stream is None or isinstance(stream, int):
+        return stream
+    return stream.cuda_stream
 
 
 def lorads_op_sddmm(p, prec: int, r: int, ld: int, U, V, q, stream=None) -> int:
