@@ -113,6 +113,7 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g) {
   uint8_t* sB = smem + 128 * K * 2;
   __shared__ uint64_t bar;
   __shared__ uint32_t tmem_base;
+  __shared__ __align__(16) float bias[HID];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tile = blockIdx.x;
   const int row0 = tile * 128;
@@ -122,6 +123,8 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g) {
   else stage_rows<128, K>(g.A, g.lda, row0, g.rows, g.a_cols, sA);
   if (g.b_trans) stage_transposed<N, K>(g.B, g.ldb, g.b_rows, row0, g.rows, sB);
   else stage_rows<N, K>(g.B, g.ldb, 0, g.b_rows, g.b_cols, sB);
+  if (g.epi == EPI_LAYER && tid < HID) bias[tid] = g.bias[tid];
+  if (g.epi == EPI_HEADS && tid == 0) bias[0] = g.bias[0];
   tc::fence_proxy_async_smem();
   tc::fence_before();
   __syncthreads();
@@ -173,22 +176,34 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(GemmArgs g) {
         *reinterpret_cast<float4*>(pp + i) =
             make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
     } else if (row < g.rows) {
+      // the bias is read before anything is stored and rows go out by 16 bytes: element by element,
+      // each bias load waited behind the store before it, 40 us per layer at any size
       if (g.epi == EPI_LAYER) {
+        float v[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float s = acc[i] + g.bias[c0 + i];
-          g.out[(size_t)row * HID + c0 + i] = s;
-          g.out_h[(size_t)row * CATW + c0 + i] = __float2bfloat16(fmaxf(s, 0.f));
+        for (int i = 0; i < 16; i += 4) {
+          const float4 b = *reinterpret_cast<const float4*>(bias + c0 + i);
+          v[i] = acc[i] + b.x;
+          v[i + 1] = acc[i + 1] + b.y;
+          v[i + 2] = acc[i + 2] + b.z;
+          v[i + 3] = acc[i + 3] + b.w;
         }
-      } else if (g.epi == EPI_HEADS) {
+        float4* so = reinterpret_cast<float4*>(g.out + (size_t)row * HID + c0);
+        __align__(16) bf16 h[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int c = c0 + i;
-          g.out[(size_t)row * HEADW + c] = (c == RMAX) ? acc[i] + g.bias[0] : acc[i];
-        }
+        for (int i = 0; i < 16; ++i) h[i] = __float2bfloat16(fmaxf(v[i], 0.f));
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          so[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        uint4* ho = reinterpret_cast<uint4*>(g.out_h + (size_t)row * CATW + c0);
+        ho[0] = reinterpret_cast<const uint4*>(h)[0];
+        ho[1] = reinterpret_cast<const uint4*>(h)[1];
       } else {
+        if (g.epi == EPI_HEADS && c0 == RMAX) acc[0] += bias[0];
+        float4* o = reinterpret_cast<float4*>(g.out + (size_t)row * (g.epi == EPI_HEADS ? HEADW : g.ldo) + c0);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) g.out[(size_t)row * g.ldo + c0 + i] = acc[i];
+        for (int i = 0; i < 4; ++i)
+          o[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
       }
     }
   }
