@@ -134,7 +134,7 @@ __global__ void op_hessian_kernel(DevProblem P, int ld, T rho, T gamma, const T*
 // ---- FP64 operators.  FP64 issues one warp instruction per SM every 16 clocks whatever its lanes
 // do (1/64 of the FP32 rate), so these kernels are bound by the FP64 instructions they issue, and
 // the layout keeps those few: a row of ld doubles is ld / 2 units of 16 bytes, dealt to G lanes (lane
-// l: units l, l + G, ...), N units per lane with G the smallest power of two that gives N <= 8.  The
+// l: units l, l + G, ...), N <= 8 units per lane (unit_lanes).  The
 // solver's layout (4-element chunks, two per lane) leaves a third of the lanes of a ld = 20 row
 // without elements in instructions that are issued all the same.
 struct UnitRow {
@@ -435,15 +435,19 @@ struct Launch {
 LORADS_DECLARE_LAUNCH(double)
 LORADS_DECLARE_LAUNCH(float)
 
-// lanes per row and units per lane of the FP64 operators (ld <= 256: at most 16 lanes)
-inline int unit_lanes(int ld) {
-  int G = 1;
+// lanes per row and units per lane of the FP64 operators (ld <= 256): the fewest lanes that leave at
+// most 8 units each, which issue the fewest FP64 instructions; up to 8 where
+// the rows alone would not fill the SMs with 16 warps and latency counts instead (2 lanes per row
+// took 29 us for a product that 8 lanes form in 14)
+inline int unit_lanes(int ld, long long rows) {
+  int G = 2;
   while ((ld / 2 + G - 1) / G > 8) G <<= 1;
-  return G < 2 ? 2 : G;
+  while (G < 8 && 2 * G <= ld / 2 && rows * G < 152LL * 512) G <<= 1;
+  return G;
 }
 template <template <int> class K, class... A>
-inline cudaError_t launch_units(int ld, A... args) {
-  const int G = unit_lanes(ld);
+inline cudaError_t launch_units(int ld, long long rows, A... args) {
+  const int G = unit_lanes(ld, rows);
   switch ((ld / 2 + G - 1) / G) {
     case 1: K<1>::go(G, args...); break;
     case 2: K<2>::go(G, args...); break;
@@ -482,7 +486,7 @@ struct HessianF64Diag {
   template <>                                                                                  \
   cudaError_t Launch<T>::op_sddmm(const DevProblem& P, int ld, const T* U, const T* V,         \
                                   double* q, int grid, cudaStream_t s) {                       \
-    if constexpr (sizeof(T) == 8) return launch_units<SddmmF64>(ld, grid, s, P, ld, U, V, q);  \
+    if constexpr (sizeof(T) == 8) return launch_units<SddmmF64>(ld, P.m, grid, s, P, ld, U, V, q);  \
     else op_sddmm_kernel<T><<<grid, 256, 0, s>>>(P, ld, U, V, q);                              \
     return cudaGetLastError();                                                                 \
   }                                                                                            \
@@ -490,7 +494,7 @@ struct HessianF64Diag {
   cudaError_t Launch<T>::op_spmm(const DevProblem& P, int ld, const double* w, double gamma,   \
                                  const T* V, T* out, int grid, cudaStream_t s) {               \
     if constexpr (sizeof(T) == 8) {                                                            \
-      if (P.a_diag_only) return launch_units<SpmmF64Diag>(ld, grid, s, P, ld, w, gamma, V, out); \
+      if (P.a_diag_only) return launch_units<SpmmF64Diag>(ld, P.n, grid, s, P, ld, w, gamma, V, out); \
     }                                                                                          \
     op_spmm_kernel<T><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);                           \
     return cudaGetLastError();                                                                 \
@@ -506,7 +510,7 @@ struct HessianF64Diag {
     } else if (!P.a_diag_only) {                                                               \
       op_hessian_kernel<T><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, out);          \
     } else if constexpr (sizeof(T) == 8) {                                                     \
-      return launch_units<HessianF64Diag>(ld, grid, s, P, ld, rho, gamma, V, Pm, out);         \
+      return launch_units<HessianF64Diag>(ld, P.n, grid, s, P, ld, rho, gamma, V, Pm, out);         \
     } else {                                                                                   \
       op_hessian_diag_kernel<T><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, out);     \
     }                                                                                          \

@@ -1234,7 +1234,7 @@ struct Solver {
     }
     Frag<T> rt, wt, gt;
     frag_convert(rt, accR);
-    const T at = (T)c.a;                          // = rowa<T>(P)[j] (0 without a constraint)
+    const T at = from_double<T>(c.a);                          // = rowa<T>(P)[j] (0 without a constraint)
     if (dout != nullptr) {
       const T sa = (T)rho * at * at;
       const T c = sa / ((T)gamma + sa * frag_dot(Wjt, Wjt, tm));
@@ -1251,7 +1251,7 @@ struct Solver {
     frag_store(rt, A.R, j, ld, tm);
     frag_store(wt, A.HP, j, ld, tm);
     gt = rt;
-    frag_axpy(gt, (T)cg, Wjt);
+    frag_axpy(gt, from_double<T>(cg), Wjt);
     const double d1 = to_double(frag_dot(rt, rt, tm)), d2 = to_double(frag_dot(wt, rt, tm));
     const double d3 = to_double(frag_dot(gt, gt, tm));
     if (tm.lead) {
@@ -1933,7 +1933,7 @@ struct Solver {
     Frag<T> Uj;
     frag_load(Uj, A.Ut, j, ld, tm);
     const T u2 = frag_dot(Uj, Uj, tm);
-    const T mu = (T)A.e[j];
+    const T mu = from_double<T>(A.e[j]);
 #pragma unroll
     for (int k = 0; k < KMAX; ++k)
 #pragma unroll
@@ -1986,7 +1986,7 @@ struct Solver {
       frag_load(Uj, Us, j, ld, tm);
       frag_load(r, Rb[0], j, ld, tm);
       const T u2 = frag_dot(Uj, Uj, tm);
-      sphere_hess_row(j, Rb[0], r, Uj, u2, (T)A.e[j], tm, w);
+      sphere_hess_row(j, Rb[0], r, Uj, u2, from_double<T>(A.e[j]), tm, w);
       frag_store(w, Wb[0], j, ld, tm);
       const double d1 = to_double(frag_dot(r, r, tm)), d2 = to_double(frag_dot(w, r, tm));
       if (tm.lead) {
@@ -2102,7 +2102,7 @@ struct Solver {
           frag_load(Uj, Us, j, ld, tm);
           frag_load(r, Rb[cur], j, ld, tm);
           const T u2 = frag_dot(Uj, Uj, tm);
-          sphere_hess_row(j, Rb[cur], r, Uj, u2, (T)A.e[j], tm, w);
+          sphere_hess_row(j, Rb[cur], r, Uj, u2, from_double<T>(A.e[j]), tm, w);
           frag_store(w, Wb[cur], j, ld, tm);
           const T d1 = frag_dot(r, r, tm), d2 = frag_dot(w, r, tm);
           pair_add(d1, d2, tm, z0, z1);
@@ -2137,7 +2137,7 @@ struct Solver {
       frag_load(Uj, A.Ut, j, ld, tm);
       frag_load(dj, A.Dl, j, ld, tm);
       const T u2 = frag_dot(Uj, Uj, tm);
-      sphere_hess_row(j, A.Dl, dj, Uj, u2, (T)A.e[j], tm, w);
+      sphere_hess_row(j, A.Dl, dj, Uj, u2, from_double<T>(A.e[j]), tm, w);
       frag_load(gj, A.grad, j, ld, tm);
       frag_convert(dd, dj);
       const double a1 = frag_dot(gj, dd, tm), a2 = to_double(frag_dot(dj, w, tm));
