@@ -652,11 +652,13 @@ __device__ __forceinline__ void hessian_row(T a, const Frag<T>& Wj, const Frag<T
                                             T gamma, const Team& t, Frag<T>& out) {
   const T q = a * frag_dot(Pj, Wj, t);
   const T aq = a * q;
+  // a row without a constraint takes no term from W (0 times an Inf there would be NaN)
+  const bool on = a != T(0);
 #pragma unroll
   for (int kk = 0; kk < KMAX; ++kk)
 #pragma unroll
     for (int ee = 0; ee < CHUNK; ++ee)
-      out.v[kk][ee] = fma(rho, aq * Wj.v[kk][ee], gamma * Pj.v[kk][ee]);
+      out.v[kk][ee] = fma(rho, on ? aq * Wj.v[kk][ee] : T(0), gamma * Pj.v[kk][ee]);
 }
 
 // (A^T(w) - C) W on row j, w_i = wb * b_i + wl * lambda_i + we * e_i (e may be NULL),
@@ -784,8 +786,9 @@ __device__ __forceinline__ void frag_warp_combine(Frag<T>& f, int G) {
 }
 
 // (H P)_j = rho sum a q W_k + gamma P_j with the whole warp; out valid in every lane.  All
-// sub-teams take the same number of rounds, two entries each; an entry past the end of the row has
-// a = 0 and reads nothing.  A diagonal entry (k = j) takes P_k = 0: q = a P_j . W_j.
+// sub-teams take the same number of rounds, two entries each; an entry past the end of the row reads
+// and adds nothing.  A diagonal entry (k = j) has the one product q = a P_j . W_j.  (Adding products
+// with zero rows instead would turn an Inf of the other factor into NaN.)
 template <typename T>
 __device__ void hessian_row_warp(const DevProblem& P, const T* Wm, const T* Pm, int ld, int j,
                                  const Frag<T>& Pj, T rho, T gamma, const WarpRow& w,
@@ -799,27 +802,34 @@ __device__ void hessian_row_warp(const DevProblem& P, const T* Wm, const T* Pm, 
   for (int e0 = P.A_rp[j]; e0 < e1; e0 += 2 * w.S) {
     Frag<T> Wk[2], Pk[2];
     T a[2], q[2];
+    bool on[2], off[2];               // an entry of the row; off the diagonal
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int e = e0 + w.sub + h * w.S;
       Team tw = t, tp = t;
       int k = j;
       a[h] = T(0);
-      if (e < e1) {
+      on[h] = e < e1;
+      if (on[h]) {
         k = P.A_col[e];
         a[h] = av[e];
       } else {
         tw.nc = 0;
       }
-      tp.nc = k == j ? 0 : tw.nc;
+      off[h] = k != j;
+      tp.nc = off[h] ? tw.nc : 0;
       frag_load(Wk[h], Wm, k, ld, tw);
       frag_load(Pk[h], Pm, k, ld, tp);
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-      q[h] = a[h] * team_sum(frag_dot_local(Pj, Wk[h]) + frag_dot_local(Pk[h], Wj), t);
+    for (int h = 0; h < 2; ++h) {
+      T loc = frag_dot_local(Pj, Wk[h]);
+      if (off[h]) loc += frag_dot_local(Pk[h], Wj);
+      q[h] = a[h] * team_sum(loc, t);
+    }
 #pragma unroll
-    for (int h = 0; h < 2; ++h) frag_axpy(acc, a[h] * q[h], Wk[h]);
+    for (int h = 0; h < 2; ++h)
+      if (on[h]) frag_axpy(acc, a[h] * q[h], Wk[h]);
   }
   frag_warp_combine(acc, t.G);
 #pragma unroll

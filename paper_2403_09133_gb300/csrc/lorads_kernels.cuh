@@ -214,6 +214,8 @@ __global__ void __launch_bounds__(256) op_spmm_f64_diag_kernel(DevProblem P, int
   for (int j = t.id; j < P.n; j += t.count) {
     const int con = P.row_con[j];
     const double own = con >= 0 ? fma(P.row_a[j], w[con], gamma) : gamma;
+    // V_j enters only with a constraint or a gamma (0 times an Inf there would be NaN)
+    const int own_units = con >= 0 || gamma != 0.0 ? t.units : 0;
     double2 acc[N];
 #pragma unroll
     for (int u = 0; u < N; ++u) acc[u] = make_double2(0.0, 0.0);
@@ -244,7 +246,7 @@ __global__ void __launch_bounds__(256) op_spmm_f64_diag_kernel(DevProblem P, int
 #pragma unroll
     for (int u = 0; u < N; ++u)
       if (t.lane + G * u < t.units) {
-        const double2 x = unit_at(V + (size_t)j * ld, t.lane + G * u, t.units);
+        const double2 x = unit_at(V + (size_t)j * ld, t.lane + G * u, own_units);
         *reinterpret_cast<double2*>(out + (size_t)j * ld + 2 * (t.lane + G * u)) =
             make_double2(fma(own, x.x, acc[u].x), fma(own, x.y, acc[u].y));
       }
@@ -273,7 +275,12 @@ __global__ void __launch_bounds__(256) op_hessian_f64_diag_kernel(DevProblem P, 
       y = fma(p[u].y, v[u].y, y);
     }
     __syncwarp();
-    const double c = rho * (a * (a * team_sum64(x + y, G)));
+    double c = rho * (a * (a * team_sum64(x + y, G)));
+    if (a == 0.0) {                  // no constraint: nothing of V, whatever it holds
+      c = 0.0;
+#pragma unroll
+      for (int u = 0; u < N; ++u) v[u] = make_double2(0.0, 0.0);
+    }
     if (live) {
 #pragma unroll
       for (int u = 0; u < N; ++u)
