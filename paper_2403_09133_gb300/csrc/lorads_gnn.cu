@@ -17,6 +17,7 @@
 
 #include "../../include/lorads.h"
 #include "lorads_device.cuh"
+#include "lorads_fetch.h"
 #include "lorads_gemm_tc.cuh"
 
 using bf16 = __nv_bfloat16;
@@ -767,12 +768,13 @@ int lorads_gnn_forward(lorads_gnn* g, int32_t r, double* U0, double* y0, void* s
   double* const yd = Ud + (size_t)n * r;
   int st = forward_impl(g, r, s, Ud, yd);
   if (st != LORADS_OK) return st;
-  int herr = 0;
-  if (U0) GCU(cudaMemcpyAsync(U0, Ud, sizeof(double) * n * r, cudaMemcpyDeviceToHost, s));
-  if (y0) GCU(cudaMemcpyAsync(y0, yd, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
-  GCU(cudaMemcpyAsync(&herr, g->err, 4, cudaMemcpyDeviceToHost, s));
-  GCU(cudaStreamSynchronize(s));
-  return herr ? LORADS_ERR_DEVICE : LORADS_OK;
+  const FetchItem items[] = {{U0, Ud, sizeof(double) * n * r}, {y0, yd, sizeof(double) * n}};
+  return fetch_outputs(
+      g->err, items, 2, LORADS_ERR_DEVICE,
+      [s](void* dst, const void* src, size_t bytes) {
+        return cuda_status(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s));
+      },
+      [s] { return cuda_status(cudaStreamSynchronize(s)); });
 }
 
 int lorads_gnn_train_step(lorads_gnn* g, int32_t r, const double* Xs, const double* ys, double lr,
