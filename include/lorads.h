@@ -117,9 +117,14 @@ typedef struct lorads_params {
   double time_limit_s;     /* wall-clock cap of one solve on the device (60 s)               */
   int32_t threads;         /* CTA size of the solver kernels, a multiple of 32, >= 128:     */
                            /*    <= 384 for one-CTA solves and batches, <= 320 for the grid  */
-                           /*    scope                                                        */
+                           /*    scope (a library-chosen grid is one CTA for 352 and 384 up  */
+                           /*    to n = 511)                                                  */
                            /*    (0 = library choice; batches autotune 128, 256, 384)         */
-  int32_t grid;            /* solver CTAs (0 = library choice; 1 forces one-CTA scope)       */
+  int32_t grid;            /* solver CTAs (0 = library choice: one CTA below n = 512, in the  */
+                           /*    FP64 form below n = 256 when every constraint is one diagonal */
+                           /*    entry and below n = 40 otherwise, more from there; 1 forces  */
+                           /*    one-CTA scope, the geometry of a batch's problems in groups  */
+                           /*    of one CTA)                                                   */
   int32_t team_mult;       /* lanes per factor row = team_mult x the minimum for the rank    */
                            /* (1, 2, 4, 8; 0 = 1, or autotuned by lorads_solve_batch)         */
   int32_t kkt_dinf;        /* 1: the final test includes the dual measure                    */

@@ -719,16 +719,9 @@ static void record_solution(lorads_problem* p, const SolveOut& out, const lorads
   p->has_solution = out.ld > 0;
 }
 
-// Launch geometry of a single-problem solve: one CTA for small problems, the whole GPU from a few
-// hundred rows up (n >= 512).  The FP64 form goes over earlier, since one SM's FP64 unit (a warp
-// instruction every 16 clocks) bounds it: from n = 256 with diagonal constraints (60 iterations on
-// ER graphs of degree 6, one CTA / 152: n = 200 9.5 / 10.3 ms, 256 10.4 / 10.5, 320 22.7 / 11.5, 500 31.9 /
-// 11.5), and from n = 40 in the general form, whose rows carry many entries (matrix completion n = 60
-// 42.5 / 12.7 ms, 400 338 / 15; theta n = 20 31.5 / 34.4, 40 28.5 / 23.9).  The mixed form stays on one
-// CTA below 512: another geometry sums in another order, and its FP32 iterates then differ by far
-// more than rounding.  One-CTA solves take prm->threads (default SOLVER_THREADS);
-// whole-GPU solves take prm->threads or, by default, enough teams for one row each at the
-// initial rank, within [128, 320] threads, and at most as many CTAs as are co-resident.
+// Launch geometry of a single-problem solve.  One-CTA solves take prm->threads (default
+// SOLVER_THREADS); whole-GPU solves take prm->threads or, by default, enough teams for one row each at
+// the initial rank, within [128, 320] threads, and at most as many CTAs as are co-resident.
 // lorads_solve and lorads_solve_static both launch with it, so that the same parameters
 // give the same reduction order and iterates on either path.
 template <typename T>
@@ -736,10 +729,8 @@ static int solve_geometry(const lorads_problem* p, const lorads_params* prm,
                           const DevParams& dv, int dev_sms, bool* whole_gpu, int* grid_out,
                           int* threads_out) {
   int grid = prm->grid;
-  if (grid <= 0) {
-    const int64_t whole_from = sizeof(T) == 4 ? 512 : (p->dp.a_diag_only ? 256 : 40);
-    grid = p->n < whole_from ? 1 : dev_sms;
-  }
+  if (grid <= 0)
+    grid = default_ctas({p->n, sizeof(T) == 8, p->dp.a_diag_only != 0, prm->threads, dev_sms});
   *whole_gpu = grid != 1;
   if (grid == 1) {
     const int threads = prm->threads > 0 ? prm->threads : SOLVER_THREADS;

@@ -1,14 +1,10 @@
 // Kernel entry points of the solver and of the operator calls, instantiated per element
 // type by lorads_f64.cu / lorads_f32.cu.
 #pragma once
+#include "lorads_geometry.h"
 #include "lorads_solver.cuh"
 
 namespace lorads {
-
-constexpr int SOLVER_THREADS = 256;       // one-CTA solver: default CTA size ...
-constexpr int BLOCK_THREADS_MAX = 384;    // ... and the largest (batches autotune 128..384)
-constexpr int GRID_THREADS_MAX = 320;     // grid solver: CTA size chosen per problem
-constexpr int SOLVER_THREADS_MIN = 128;   // every solver CTA: four warps, one per Lanczos chain
 
 // one CTA per problem; CTAs take problems from a queue (batches), or a single problem
 template <typename T, int SUB>

@@ -1,0 +1,59 @@
+"""The library's choice of CTAs for a single solve (csrc/lorads_geometry.h), compiled for the host."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2403_09133_gb300", "csrc")
+
+PROGRAM = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "lorads_geometry.h"
+int main(int argc, char** argv) {
+  for (int i = 1; i + 4 < argc; i += 5) {
+    lorads::SolveSize s{};
+    s.n = atol(argv[i]);
+    s.fp64 = atoi(argv[i + 1]) != 0;
+    s.diag_only = atoi(argv[i + 2]) != 0;
+    s.threads = atoi(argv[i + 3]);
+    s.sms = atoi(argv[i + 4]);
+    std::printf("%d\n", lorads::default_ctas(s));
+  }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def ctas(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no g++")
+    d = tmp_path_factory.mktemp("geometry")
+    (d / "g.cpp").write_text(PROGRAM)
+    subprocess.run([cxx, "-O1", "-std=c++17", "-I", CSRC, str(d / "g.cpp"), "-o", str(d / "g")],
+                   check=True)
+
+    def run(cases):
+        args = [str(int(x)) for c in cases for x in c]
+        out = subprocess.run([str(d / "g"), *args], capture_output=True, text=True, check=True)
+        return list(map(int, out.stdout.split()))
+    return run
+
+
+def test_a_cta_size_of_the_one_cta_kernel_keeps_small_solves_there(ctas):
+    """352 and 384 threads fit only the one-CTA kernel: below n = 512 they choose it, in both forms."""
+    cases = [(n, fp64, diag, th, 152) for n in (1, 39, 40, 60, 255, 256, 300, 511)
+             for fp64 in (0, 1) for diag in (0, 1) for th in (352, 384)]
+    assert ctas(cases) == [1] * len(cases)
+
+
+def test_thresholds(ctas):
+    one = [(39, 1, 0, 0, 152), (255, 1, 1, 0, 152), (511, 0, 0, 0, 152), (511, 0, 1, 0, 152)]
+    assert ctas(one) == [1] * len(one)
+    more = [(40, 1, 0, 0, 152), (40, 1, 0, 320, 152), (256, 1, 1, 0, 152), (256, 1, 1, 320, 152)]
+    assert min(ctas(more)) > 1
+    whole = [(512, f, d, 0, 148) for f in (0, 1) for d in (0, 1)]
+    assert ctas(whole) == [148] * len(whole)
