@@ -122,9 +122,9 @@ typedef struct lorads_params {
                            /*    (0 = library choice; batches autotune 128, 256, 384)         */
   int32_t grid;            /* solver CTAs (0 = library choice: one CTA below n = 512, in the  */
                            /*    FP64 form below n = 256 when every constraint is one diagonal */
-                           /*    entry and below n = 40 otherwise, more from there; 1 forces  */
-                           /*    one-CTA scope, the geometry of a batch's problems in groups  */
-                           /*    of one CTA)                                                   */
+                           /*    entry and below n = 40 otherwise; from there the CTAs that   */
+                           /*    the rows fill, and all SMs from n = 512; 1 forces one-CTA    */
+                           /*    scope, the geometry of a batch's problems in groups of one)  */
   int32_t team_mult;       /* lanes per factor row = team_mult x the minimum for the rank    */
                            /* (1, 2, 4, 8; 0 = 1, or autotuned by lorads_solve_batch)         */
   int32_t kkt_dinf;        /* 1: the final test includes the dual measure                    */

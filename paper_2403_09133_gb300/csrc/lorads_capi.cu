@@ -729,8 +729,12 @@ static int solve_geometry(const lorads_problem* p, const lorads_params* prm,
                           const DevParams& dv, int dev_sms, bool* whole_gpu, int* grid_out,
                           int* threads_out) {
   int grid = prm->grid;
-  if (grid <= 0)
-    grid = default_ctas({p->n, sizeof(T) == 8, p->dp.a_diag_only != 0, prm->threads, dev_sms});
+  if (grid <= 0) {
+    const int rmax = std::max(dv.rank_cap, dv.phase1 ? 0 : p->start_r);
+    const int lanes = std::min(team_size_for(round4(rmax)) * dv.team_mult, 32);
+    grid = default_ctas(
+        {p->n, sizeof(T) == 8, p->dp.a_diag_only != 0, lanes, prm->threads, dev_sms});
+  }
   *whole_gpu = grid != 1;
   if (grid == 1) {
     const int threads = prm->threads > 0 ? prm->threads : SOLVER_THREADS;

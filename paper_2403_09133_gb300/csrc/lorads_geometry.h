@@ -13,22 +13,39 @@ struct SolveSize {
   int64_t n;          // rows
   bool fp64;          // the plain FP64 form (else the mixed form)
   bool diag_only;     // every constraint one diagonal entry, at most one per row
+  int lanes;          // lanes of a factor row at the largest rank
   int threads;        // the caller's CTA size; 0: library choice
   int sms;
 };
 
 // One CTA for small problems, the whole GPU from a few hundred rows up (n >= 512).  The FP64 form
-// goes over earlier, since one SM's FP64 unit (a warp instruction every 16 clocks) bounds it: from
-// n = 256 with diagonal constraints (60 iterations on ER graphs of degree 6, one CTA / 152: n = 200
-// 9.5 / 10.3 ms, 256 10.4 / 10.5, 320 22.7 / 11.5, 500 31.9 / 11.5), and from n = 40 in the general form,
-// whose rows carry many entries (matrix completion n = 60 42.5 / 12.7 ms, 400 338 / 15; theta n = 20
-// 31.5 / 34.4, 40 28.5 / 23.9).  The mixed form stays on one CTA below 512: another geometry sums in
-// another order, and its FP32 iterates then differ by far more than rounding.  A CTA size that only
-// the one-CTA kernel takes keeps a solve of fewer than 512 rows there.
+// leaves one CTA earlier, since one SM's FP64 unit (a warp instruction every 16 clocks) bounds it: from
+// n = 256 with diagonal constraints and from n = 40 in the general form, whose rows carry many
+// entries.  It takes the CTAs that its rows fill and no more, a team of lanes per row with diagonal
+// constraints and a warp per row in the general form: further CTAs only wait at the barriers, and they
+// keep other callers' solves off the GPU.  Measured (ms, grids of 1 / 8 / 16 / 32 / 76 / 152):
+//   ER degree 6, 60 iterations      n = 256   10.4  10.2  10.3  10.3  10.4  10.4
+//                                   n = 300   21.2  10.4  10.3  10.3  10.5  10.7
+//                                   n = 511   32.1  11.3  11.3  11.2  11.4  11.6
+//   the same, row-block direct      n = 511   21.2   8.7   8.7   8.6   8.7   8.9
+//   completion, 15 iterations       n = 60    42.5  15.7  12.4  12.4  12.6  13.0
+//                                   n = 200    157  36.4  24.4  16.5  12.7  13.2
+//                                   n = 500    329  79.3  47.6  32.4  25.3  22.1
+//   theta, 15 iterations            n = 20    31.5  33.6  33.6  33.8  34.0  34.6
+//                                   n = 40    24.6  21.0  19.8  19.7  19.8  19.7
+// Eight callers side by side, a thread, stream and problem each (solves a second, grids of 1 / 8 /
+// 16 / 152): ER n = 256 705 / 714 / 712 / 169, n = 500 238 / 651 / 646 / 158; completion n = 60
+// 108 / 270 / 328 / 148, n = 400 19 / 99 / 163 / 121 (on one CTA each, completions of n = 400 overtake
+// a grid of 100 at about 50 callers).  The mixed form stays on one CTA below 512: another geometry
+// sums in another order, and its FP32 iterates then differ by far more than rounding.  A CTA size
+// that only the one-CTA kernel takes keeps a solve of fewer than 512 rows there.
 inline int default_ctas(const SolveSize& p) {
   if (p.n >= 512) return p.sms;
   if (!p.fp64 || p.n < (p.diag_only ? 256 : 40) || p.threads > GRID_THREADS_MAX) return 1;
-  return p.sms;
+  const int64_t lanes = p.n * (p.diag_only ? p.lanes : 32);
+  const int64_t threads = p.threads > 0 ? p.threads : SOLVER_THREADS_MIN;
+  const int64_t ctas = (lanes + threads - 1) / threads;
+  return (int)(ctas < 2 ? 2 : ctas > p.sms ? p.sms : ctas);
 }
 
 }  // namespace lorads

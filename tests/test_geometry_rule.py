@@ -13,13 +13,14 @@ PROGRAM = r"""
 #include <cstdlib>
 #include "lorads_geometry.h"
 int main(int argc, char** argv) {
-  for (int i = 1; i + 4 < argc; i += 5) {
+  for (int i = 1; i + 5 < argc; i += 6) {
     lorads::SolveSize s{};
     s.n = atol(argv[i]);
     s.fp64 = atoi(argv[i + 1]) != 0;
     s.diag_only = atoi(argv[i + 2]) != 0;
     s.threads = atoi(argv[i + 3]);
     s.sms = atoi(argv[i + 4]);
+    s.lanes = atoi(argv[i + 5]);
     std::printf("%d\n", lorads::default_ctas(s));
   }
 }
@@ -37,7 +38,7 @@ def ctas(tmp_path_factory):
                    check=True)
 
     def run(cases):
-        args = [str(int(x)) for c in cases for x in c]
+        args = [str(int(x)) for c in cases for x in (*c, 4)[:6]]
         out = subprocess.run([str(d / "g"), *args], capture_output=True, text=True, check=True)
         return list(map(int, out.stdout.split()))
     return run
@@ -57,3 +58,16 @@ def test_thresholds(ctas):
     assert min(ctas(more)) > 1
     whole = [(512, f, d, 0, 148) for f in (0, 1) for d in (0, 1)]
     assert ctas(whole) == [148] * len(whole)
+
+
+def test_no_more_ctas_than_the_rows_fill(ctas):
+    """From the thresholds to n = 511 an FP64 solve takes the CTAs that its rows fill: with fewer rows than
+    that many SMs hold, callers side by side share the GPU."""
+    diag = [(n, 1, 1, th, 152, lanes) for n in (256, 257, 300, 511) for th in (0, 128, 256, 320)
+            for lanes in (1, 2, 4, 8, 32)]
+    want = [max(2, min(152, -(-n * lanes // (th or 128)))) for n, _, _, th, _, lanes in diag]
+    assert ctas(diag) == want
+    general = [(n, 1, 0, threads, 152) for n in (40, 41, 60, 120, 400, 511) for threads in (0, 320)]
+    want = [max(2, min(152, -(-n * 32 // (th or 128)))) for n, _, _, th, _ in general]
+    assert ctas(general) == want
+    assert ctas([(511, 1, 0, 0, 100)]) == [100]
