@@ -730,19 +730,59 @@ __device__ __forceinline__ double sddmm_entry(const T* Um, const T* Vm, int ld, 
   return a * to_double(team_sum(loc, t));
 }
 
-// <A_i, U V^T>: the sum over constraint i's entries (team-cooperative; called by whole warps, whose
-// teams take as many rounds as the longest of their constraints)
+// <A_i, U V^T> where every constraint has one entry (the i-th entry is constraint i's)
 template <typename T>
 __device__ __forceinline__ double sddmm_con(const DevProblem& P, const T* Um, const T* Vm, int ld,
                                             int i, const Team& t) {
+  return sddmm_entry<T>(Um, Vm, ld, P.con_r[i], P.con_c[i], P.con_a[i], t);
+}
+
+// <A_i, U V^T>: the sum over constraint i's entries (team-cooperative; called by whole warps, whose
+// teams take as many rounds as the longest of their constraints), two entries a round, the rows of
+// both read before either is summed.  A team that has no entry left takes part empty-handed: repeating
+// one of its own cost the warp that entry's loads and, off the diagonal, a second product in every
+// round.  Bound by the latency of the rows' loads: the trace of n = 3,000 beside 9,000 constraints of one
+// entry, FP32, r = 9, 1,507 us with repeated entries, 975 so.
+template <typename T>
+__device__ __forceinline__ double sddmm_con_multi(const DevProblem& P, const T* Um, const T* Vm,
+                                                  int ld, int i, const Team& t) {
   const int e0 = P.con_ptr[i], cnt = t.live ? P.con_ptr[i + 1] - e0 : 0;
-  const int rounds = P.a_multi ? __reduce_max_sync(0xffffffffu, cnt) : 1;
+  const int rounds = __reduce_max_sync(0xffffffffu, cnt);
   double s = 0.0;
-  for (int k = 0; k < rounds; ++k) {
-    const bool on = k < cnt;
-    const int e = on ? e0 + k : e0;
-    const double x = sddmm_entry<T>(Um, Vm, ld, P.con_r[e], P.con_c[e], P.con_a[e], t);
-    if (on) s += x;
+  for (int k = 0; k < rounds; k += 2) {
+    Frag<T> Ur[2], Vc[2];
+    int r[2], c[2];
+    double a[2];
+    T loc[2];
+    Team te[2] = {t, t};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const bool on = k + h < cnt;
+      const int e = on ? e0 + k + h : e0;
+      c[h] = P.con_c[e];
+      r[h] = on ? P.con_r[e] : c[h];
+      a[h] = P.con_a[e];
+      te[h].nc = on ? t.nc : 0;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      frag_load(Ur[h], Um, r[h], ld, te[h]);
+      frag_load(Vc[h], Vm, c[h], ld, te[h]);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) loc[h] = frag_dot_local(Ur[h], Vc[h]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (r[h] != c[h]) {
+        frag_load(Ur[h], Um, c[h], ld, te[h]);
+        frag_load(Vc[h], Vm, r[h], ld, te[h]);
+        loc[h] += frag_dot_local(Ur[h], Vc[h]);
+      }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const double x = a[h] * to_double(team_sum(loc[h], t));
+      if (k + h < cnt) s += x;
+    }
   }
   return s;
 }

@@ -68,11 +68,12 @@ solve_group_kernel(const SolverArgs<T>* args, int count, int* queue, GridCtl* ct
 }
 
 // ---- operators on caller-owned device arrays ----
-template <typename T>
+template <typename T, bool MULTI>
 __global__ void op_sddmm_kernel(DevProblem P, int ld, const T* U, const T* V, double* q) {
   const Team t = make_team(ld, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
   for (TeamRows rows(t, P.m); rows.more(); rows.next()) {
-    const double v = sddmm_con<T>(P, U, V, ld, rows.j, rows.t);
+    const double v = MULTI ? sddmm_con_multi<T>(P, U, V, ld, rows.j, rows.t)
+                           : sddmm_con<T>(P, U, V, ld, rows.j, rows.t);
     if (rows.t.lead) q[rows.j] = v;
   }
 }
@@ -154,8 +155,10 @@ __device__ __forceinline__ double team_sum64(double x, int G) {
   return x;
 }
 
-// <A_i, U V^T>: one team per constraint
-template <int N>
+// <A_i, U V^T>: one team per constraint.  MULTI: constraints of several entries, in as many rounds as
+// the longest of the warp's teams has, a team without an entry left empty-handed (see
+// sddmm_con_multi; the trace of n = 3,000, r = 9: 2,158 us with repeated entries, 1,671 so)
+template <int N, bool MULTI>
 __global__ void __launch_bounds__(256) op_sddmm_f64_kernel(DevProblem P, int ld, int G,
                                                            const double* U, const double* V,
                                                            double* q) {
@@ -164,13 +167,18 @@ __global__ void __launch_bounds__(256) op_sddmm_f64_kernel(DevProblem P, int ld,
   for (int i0 = t.id - sub; i0 < P.m; i0 += t.count) {
     const bool live = i0 + sub < P.m;
     const int i = live ? i0 + sub : P.m - 1;
-    const int e0 = P.con_ptr[i], cnt = live ? P.con_ptr[i + 1] - e0 : 0;
-    const int rounds = P.a_multi ? __reduce_max_sync(0xffffffffu, cnt) : 1;
+    int e0 = i, cnt = 1, rounds = 1;
+    if (MULTI) {
+      e0 = P.con_ptr[i];
+      cnt = live ? P.con_ptr[i + 1] - e0 : 0;
+      rounds = __reduce_max_sync(0xffffffffu, cnt);
+    }
     double s = 0.0;
     for (int k = 0; k < rounds; ++k) {
-      const int e = k < cnt ? e0 + k : e0;
-      const int r = P.con_r[e], c = P.con_c[e];
+      const bool on = !MULTI || k < cnt;
+      const int e = on ? e0 + k : e0, c = P.con_c[e], r = on ? P.con_r[e] : c;
       const double a = P.con_a[e];
+      const int units = on ? t.units : 0;
       const double* Ur = U + (size_t)r * ld;
       const double* Vc = V + (size_t)c * ld;
       const double* Uc = U + (size_t)c * ld;
@@ -178,23 +186,23 @@ __global__ void __launch_bounds__(256) op_sddmm_f64_kernel(DevProblem P, int ld,
       double x = 0.0, y = 0.0;
 #pragma unroll
       for (int u = 0; u < N; ++u) {
-        const double2 p = unit_at(Ur, t.lane + G * u, t.units);
-        const double2 v = unit_at(Vc, t.lane + G * u, t.units);
+        const double2 p = unit_at(Ur, t.lane + G * u, units);
+        const double2 v = unit_at(Vc, t.lane + G * u, units);
         x = fma(p.x, v.x, x);
         y = fma(p.y, v.y, y);
       }
       if (r != c) {
 #pragma unroll
         for (int u = 0; u < N; ++u) {
-          const double2 p = unit_at(Uc, t.lane + G * u, t.units);
-          const double2 v = unit_at(Vr, t.lane + G * u, t.units);
+          const double2 p = unit_at(Uc, t.lane + G * u, units);
+          const double2 v = unit_at(Vr, t.lane + G * u, units);
           x = fma(p.x, v.x, x);
           y = fma(p.y, v.y, y);
         }
       }
       __syncwarp();
       x = a * team_sum64(x + y, G);
-      if (k < cnt) s += x;
+      if (on) s += x;
     }
     if (live && t.lane == 0) q[i] = s;
   }
@@ -467,7 +475,8 @@ template <int N>
 struct SddmmF64 {
   static void go(int G, int grid, cudaStream_t s, const DevProblem& P, int ld, const double* U,
                  const double* V, double* q) {
-    op_sddmm_f64_kernel<N><<<grid, 256, 0, s>>>(P, ld, G, U, V, q);
+    if (P.a_multi) op_sddmm_f64_kernel<N, true><<<grid, 256, 0, s>>>(P, ld, G, U, V, q);
+    else op_sddmm_f64_kernel<N, false><<<grid, 256, 0, s>>>(P, ld, G, U, V, q);
   }
 };
 template <int N>
@@ -490,7 +499,8 @@ struct HessianF64Diag {
   cudaError_t Launch<T>::op_sddmm(const DevProblem& P, int ld, const T* U, const T* V,         \
                                   double* q, int grid, cudaStream_t s) {                       \
     if constexpr (sizeof(T) == 8) return launch_units<SddmmF64>(ld, P.m, grid, s, P, ld, U, V, q);  \
-    else op_sddmm_kernel<T><<<grid, 256, 0, s>>>(P, ld, U, V, q);                              \
+    else if (P.a_multi) op_sddmm_kernel<T, true><<<grid, 256, 0, s>>>(P, ld, U, V, q);         \
+    else op_sddmm_kernel<T, false><<<grid, 256, 0, s>>>(P, ld, U, V, q);                       \
     return cudaGetLastError();                                                                 \
   }                                                                                            \
   template <>                                                                                  \

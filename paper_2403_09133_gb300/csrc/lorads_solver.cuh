@@ -282,10 +282,12 @@ struct Solver {
 #pragma unroll
       for (int k = 0; k < K; ++k) s[k] = 0.0;
       for (int t = 0; t < rounds; ++t) {
+        // a team without an entry left repeats its first one, without the mirror product (theta
+        // n = 600, FP64: 644 us per L-BFGS iteration with it, 609 without)
         const bool on = t < cnt;
-        const int e = on ? e0 + t : e0;
+        const int e = on ? e0 + t : e0, c = P.con_c[e], r = on ? P.con_r[e] : c;
         double x[K];
-        f(P.con_r[e], P.con_c[e], P.con_a[e], tmc, x);
+        f(r, c, P.con_a[e], tmc, x);
 #pragma unroll
         for (int k = 0; k < K; ++k)
           if (on) s[k] += x[k];
