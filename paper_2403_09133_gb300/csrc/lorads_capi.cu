@@ -429,6 +429,7 @@ static int assemble(lorads_problem* p, const DevAlloc& al) {
   dp.op_q = d_op_q;
   dp.b = d_b;
   dp.A_rp = d_A_rp;
+  dp.a_nnz = (int64_t)A_val.size();
   dp.A_col = d_A_col;
   dp.A_con = d_A_con;
   dp.A_val = d_A_val;

@@ -60,6 +60,7 @@ struct DevProblem {
   const int* A_con;
   const double* A_val;
   const float* A_valf;
+  int64_t a_nnz;   // entries of A_col
   // C as symmetric CSR over rows
   const int* C_rp;
   const int* C_col;
@@ -825,11 +826,50 @@ __device__ __forceinline__ void frag_warp_combine(Frag<T>& f, int G) {
     }
 }
 
+// H entries per sub-team of row j's terms a q W_k, from entry e0 on (all lanes of the warp).  FULL: every
+// sub-team has H; else an entry past the row's end e1 reads and adds nothing.  A diagonal entry
+// (k = j) has the one product q = a P_j . W_j.  (Adding products with zero rows instead would turn an
+// Inf of the other factor into NaN.)
+template <typename T, int H, bool FULL>
+__device__ __forceinline__ void hessian_entries(const DevProblem& P, const T* Wm, const T* Pm, int ld,
+                                                int j, int e0, int e1, const Frag<T>& Pj,
+                                                const Frag<T>& Wj, const WarpRow& w,
+                                                Frag<T>& acc) {
+  const Team& t = w.st;
+  const T* av = aval<T>(P);
+  Frag<T> Wk[H], Pk[H];
+  T a[H], q[H];
+  bool on[H], off[H];               // an entry of the row; off the diagonal
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    const int e = e0 + w.sub + h * w.S;
+    Team tw = t, tp = t;
+    int k = j;
+    a[h] = T(0);
+    on[h] = FULL || e < e1;
+    if (on[h]) {
+      k = P.A_col[e];
+      a[h] = av[e];
+    } else {
+      tw.nc = 0;
+    }
+    off[h] = k != j;
+    tp.nc = off[h] ? tw.nc : 0;
+    frag_load(Wk[h], Wm, k, ld, tw);
+    frag_load(Pk[h], Pm, k, ld, tp);
+  }
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    const T mirror = frag_dot_local(Pk[h], Wj);
+    q[h] = a[h] * team_sum(frag_dot_local(Pj, Wk[h]) + (off[h] ? mirror : T(0)), t);
+  }
+#pragma unroll
+  for (int h = 0; h < H; ++h) frag_axpy(acc, on[h] ? a[h] * q[h] : T(0), Wk[h]);
+}
+
 // (H P)_j = rho sum a q W_k + gamma P_j with the whole warp; out valid in every lane.  All
-// sub-teams take the same number of rounds, two entries each; an entry past the end of the row reads
-// and adds nothing.  A diagonal entry (k = j) has the one product q = a P_j . W_j.  (Adding products
-// with zero rows instead would turn an Inf of the other factor into NaN.)
-template <typename T>
+// sub-teams take the same number of rounds, H entries each.
+template <typename T, int H = 2>
 __device__ void hessian_row_warp(const DevProblem& P, const T* Wm, const T* Pm, int ld, int j,
                                  const Frag<T>& Pj, T rho, T gamma, const WarpRow& w,
                                  Frag<T>& out) {
@@ -837,40 +877,12 @@ __device__ void hessian_row_warp(const DevProblem& P, const T* Wm, const T* Pm, 
   Frag<T> Wj, acc;
   frag_load(Wj, Wm, j, ld, t);
   frag_zero(acc);
-  const T* av = aval<T>(P);
   const int e1 = P.A_rp[j + 1];
-  for (int e0 = P.A_rp[j]; e0 < e1; e0 += 2 * w.S) {
-    Frag<T> Wk[2], Pk[2];
-    T a[2], q[2];
-    bool on[2], off[2];               // an entry of the row; off the diagonal
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int e = e0 + w.sub + h * w.S;
-      Team tw = t, tp = t;
-      int k = j;
-      a[h] = T(0);
-      on[h] = e < e1;
-      if (on[h]) {
-        k = P.A_col[e];
-        a[h] = av[e];
-      } else {
-        tw.nc = 0;
-      }
-      off[h] = k != j;
-      tp.nc = off[h] ? tw.nc : 0;
-      frag_load(Wk[h], Wm, k, ld, tw);
-      frag_load(Pk[h], Pm, k, ld, tp);
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      T loc = frag_dot_local(Pj, Wk[h]);
-      if (off[h]) loc += frag_dot_local(Pk[h], Wj);
-      q[h] = a[h] * team_sum(loc, t);
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (on[h]) frag_axpy(acc, a[h] * q[h], Wk[h]);
-  }
+  int e0 = P.A_rp[j];
+  for (; H == 2 && e0 + 2 * w.S <= e1; e0 += 2 * w.S)
+    hessian_entries<T, 2, true>(P, Wm, Pm, ld, j, e0, e1, Pj, Wj, w, acc);
+  for (; e0 < e1; e0 += H * w.S)
+    hessian_entries<T, H, false>(P, Wm, Pm, ld, j, e0, e1, Pj, Wj, w, acc);
   frag_warp_combine(acc, t.G);
 #pragma unroll
   for (int kk = 0; kk < KMAX; ++kk)

@@ -48,4 +48,14 @@ inline int default_ctas(const SolveSize& p) {
   return (int)(ctas < 2 ? 2 : ctas > p.sms ? p.sms : ctas);
 }
 
+// Operators with a warp per row, whose 32 / G sub-teams of G lanes take an entry of the row each: whether
+// the rows of A hold at most one entry per sub-team on average (an entry off the diagonal lies in two
+// rows).  The Hessian then takes one entry a round, for longer rows two: with short ones the second
+// is mostly past the row's end, and without it two CTAs of the FP64 kernel fit an SM where one does
+// (r = 9, one / two entries a round: n = 20,000 with 6 entries a row FP64 96 / 119 us, FP32 16.5 / 18.6;
+// n = 3,000 with 133 entries FP64 84 / 69).
+inline bool short_rows(int64_t n, int64_t entries, int lanes) {
+  return entries <= n * (32 / (lanes < 32 ? lanes : 32));
+}
+
 }  // namespace lorads

@@ -115,16 +115,17 @@ op_hessian_diag_kernel(DevProblem P, int ld, T rho, T gamma, const T* V, const T
   }
 }
 
-template <typename T>
-__global__ void op_hessian_kernel(DevProblem P, int ld, T rho, T gamma, const T* V, const T* Pm,
-                                  T* out) {
+// H: entries of a round (hessian_row_warp)
+template <typename T, int H>
+__global__ void __launch_bounds__(256) op_hessian_kernel(DevProblem P, int ld, T rho, T gamma,
+                                                         const T* V, const T* Pm, T* out) {
   const WarpRow wr =
       make_warp_row(ld, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
   for (int j = wr.warp; j < P.n; j += wr.nwarps) {
-    Frag<T> Pj, H;
+    Frag<T> Pj, Hj;
     frag_load(Pj, Pm, j, ld, wr.st);
-    hessian_row_warp<T>(P, V, Pm, ld, j, Pj, rho, gamma, wr, H);
-    if (wr.sub == 0) frag_store(H, out, j, ld, wr.st);
+    hessian_row_warp<T, H>(P, V, Pm, ld, j, Pj, rho, gamma, wr, Hj);
+    if (wr.sub == 0) frag_store(Hj, out, j, ld, wr.st);
   }
 }
 
@@ -167,18 +168,16 @@ __global__ void __launch_bounds__(256) op_sddmm_f64_kernel(DevProblem P, int ld,
   for (int i0 = t.id - sub; i0 < P.m; i0 += t.count) {
     const bool live = i0 + sub < P.m;
     const int i = live ? i0 + sub : P.m - 1;
-    int e0 = i, cnt = 1, rounds = 1;
-    if (MULTI) {
-      e0 = P.con_ptr[i];
-      cnt = live ? P.con_ptr[i + 1] - e0 : 0;
-      rounds = __reduce_max_sync(0xffffffffu, cnt);
-    }
+    // (without the loop of MULTI the compiler keeps fewer loads in flight: 10^6 one-entry constraints,
+    // r = 20, 88 us against 85)
+    const int e0 = P.con_ptr[i], cnt = live ? P.con_ptr[i + 1] - e0 : 0;
+    const int rounds = P.a_multi ? __reduce_max_sync(0xffffffffu, cnt) : 1;
     double s = 0.0;
     for (int k = 0; k < rounds; ++k) {
-      const bool on = !MULTI || k < cnt;
-      const int e = on ? e0 + k : e0, c = P.con_c[e], r = on ? P.con_r[e] : c;
+      const bool on = k < cnt;
+      const int e = on ? e0 + k : e0, c = P.con_c[e], r = !MULTI || on ? P.con_r[e] : c;
       const double a = P.con_a[e];
-      const int units = on ? t.units : 0;
+      const int units = !MULTI || on ? t.units : 0;
       const double* Ur = U + (size_t)r * ld;
       const double* Vc = V + (size_t)c * ld;
       const double* Uc = U + (size_t)c * ld;
@@ -280,7 +279,10 @@ __global__ void __launch_bounds__(256) op_hessian_f64_diag_kernel(DevProblem P, 
     }
     __syncwarp();
     double c = rho * (a * (a * team_sum64(x + y, G)));
-    if (a == 0.0) {                  // no constraint: nothing of V, whatever it holds
+    // a row without a constraint takes nothing of V, whatever it holds.  Told from a's bits: an FP64
+    // comparison is one more FP64 instruction (2^20 rows of r = 20: 149 us with it)
+    const bool none = ((__double2hiint(a) & 0x7fffffff) | __double2loint(a)) == 0;
+    if (__any_sync(0xffffffffu, none) && none) {
       c = 0.0;
 #pragma unroll
       for (int u = 0; u < N; ++u) v[u] = make_double2(0.0, 0.0);
@@ -521,7 +523,10 @@ struct HessianF64Diag {
       if (e != cudaSuccess) return e;                                                          \
       op_hessian_q_kernel<T><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, P.op_q, out); \
     } else if (!P.a_diag_only) {                                                               \
-      op_hessian_kernel<T><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, out);          \
+      if (short_rows(P.n, P.a_nnz, team_size_for(ld)))                                         \
+        op_hessian_kernel<T, 1><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, out);     \
+      else                                                                                     \
+        op_hessian_kernel<T, 2><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, out);     \
     } else if constexpr (sizeof(T) == 8) {                                                     \
       return launch_units<HessianF64Diag>(ld, P.n, grid, s, P, ld, rho, gamma, V, Pm, out);         \
     } else {                                                                                   \

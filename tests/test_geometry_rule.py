@@ -1,4 +1,5 @@
-"""The library's choice of CTAs for a single solve (csrc/lorads_geometry.h), compiled for the host."""
+"""The library's choices by size (csrc/lorads_geometry.h), compiled for the host: the CTAs of a single
+solve, the operators' forms for short rows."""
 import os
 import shutil
 import subprocess
@@ -13,6 +14,10 @@ PROGRAM = r"""
 #include <cstdlib>
 #include "lorads_geometry.h"
 int main(int argc, char** argv) {
+  if (argc == 5 && argv[1][0] == 's') {
+    std::printf("%d\n", (int)lorads::short_rows(atol(argv[2]), atol(argv[3]), atoi(argv[4])));
+    return 0;
+  }
   for (int i = 1; i + 5 < argc; i += 6) {
     lorads::SolveSize s{};
     s.n = atol(argv[i]);
@@ -39,8 +44,13 @@ def ctas(tmp_path_factory):
 
     def run(cases):
         args = [str(int(x)) for c in cases for x in (*c, 4)[:6]]
-        out = subprocess.run([str(d / "g"), *args], capture_output=True, text=True, check=True)
+        return call(*args)
+
+    def call(*args):
+        out = subprocess.run([str(d / "g"), *map(str, args)], capture_output=True, text=True,
+                             check=True)
         return list(map(int, out.stdout.split()))
+    run.call = call
     return run
 
 
@@ -71,3 +81,12 @@ def test_no_more_ctas_than_the_rows_fill(ctas):
     want = [max(2, min(152, -(-n * 32 // (th or 128)))) for n, _, _, th, _ in general]
     assert ctas(general) == want
     assert ctas([(511, 1, 0, 0, 100)]) == [100]
+
+
+def test_short_rows(ctas):
+    """At most one entry per sub-team of a warp on average."""
+    for lanes in (2, 4, 8, 32, 64):
+        S = 32 // min(lanes, 32)
+        for n in (1, 20000):
+            assert ctas.call("s", n, n * S, lanes) == [1]
+            assert ctas.call("s", n, n * S + 1, lanes) == [0]
