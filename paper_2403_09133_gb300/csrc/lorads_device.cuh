@@ -890,8 +890,31 @@ __device__ void hessian_row_warp(const DevProblem& P, const T* Wm, const T* Pm, 
     for (int ee = 0; ee < CHUNK; ++ee) out.v[kk][ee] = fma(rho, acc.v[kk][ee], gamma * Pj.v[kk][ee]);
 }
 
-// (A^T(w) - C) W on row j with the whole warp (same weights as spmm_row); out in every lane
-template <typename T>
+// H entries per sub-team of a row's sum, from entry s0 of `rounds` on: lane l holds entry l's column and
+// weight
+template <typename T, int H>
+__device__ __forceinline__ void spmm_entries(const T* Wm, int ld, int s0, int rounds, int col, T c,
+                                             const WarpRow& w, Frag<T>& acc) {
+  Frag<T> Wk[H];
+  T ck[H];
+#pragma unroll
+  for (int u = 0; u < H; ++u) {
+    const int src = s0 + u * w.S + w.sub;          // < 32 when it is one of the entries
+    const int k = __shfl_sync(0xffffffffu, col, src & 31);
+    ck[u] = __shfl_sync(0xffffffffu, c, src & 31);
+    Team tw = w.st;
+    tw.nc = src < rounds ? w.st.nc : 0;
+    frag_load(Wk[u], Wm, k, ld, tw);
+  }
+#pragma unroll
+  for (int u = 0; u < H; ++u)
+    if (s0 + u * w.S + w.sub < rounds) frag_axpy(acc, ck[u], Wk[u]);
+}
+
+// (A^T(w) - C) W on row j with the whole warp (same weights as spmm_row); out in every lane.  OWN: every
+// sub-team forms the weights of its entries, for FP64, whose products outweigh them, and for short
+// rows; else the warp forms 32 at once, H rows in flight per sub-team.
+template <typename T, bool OWN = sizeof(T) == 8, int H = 2>
 __device__ void spmm_row_warp(const DevProblem& P, const T* Wm, int ld, int j, const double* lam,
                               const double* e, double wb, double wl, double we, T gamma,
                               const WarpRow& w, Frag<T>& out) {
@@ -899,15 +922,27 @@ __device__ void spmm_row_warp(const DevProblem& P, const T* Wm, int ld, int j, c
   Frag<T> acc;
   frag_zero(acc);
   const T* cv = cval<T>(P);
-  for (int q = P.C_rp[j] + w.sub; q < P.C_rp[j + 1]; q += w.S) {
-    Frag<T> Wk;
-    frag_load(Wk, Wm, P.C_col[q], ld, t);
-    frag_axpy(acc, -cv[q], Wk);
+  {
+    const int q1 = P.C_rp[j + 1];
+    int q = P.C_rp[j] + w.sub;
+    for (; q + w.S < q1; q += 2 * w.S) {
+      const int k0 = P.C_col[q], k1 = P.C_col[q + w.S];
+      const T c0 = cv[q], c1 = cv[q + w.S];
+      Frag<T> W0, W1;
+      frag_load(W0, Wm, k0, ld, t);
+      frag_load(W1, Wm, k1, ld, t);
+      frag_axpy(acc, -c0, W0);
+      frag_axpy(acc, -c1, W1);
+    }
+    if (q < q1) {
+      Frag<T> Wk;
+      frag_load(Wk, Wm, P.C_col[q], ld, t);
+      frag_axpy(acc, -cv[q], Wk);
+    }
   }
   const T* av = aval<T>(P);
   const bool a_part = (wb != 0.0) || (lam != nullptr) || (e != nullptr);
-  if (a_part && sizeof(T) == 8) {
-    // FP64: the products outweigh the weights, and four rows in flight would halve the warps
+  if (a_part && OWN) {
     const int q1 = P.A_rp[j + 1];
     int q = P.A_rp[j] + w.sub;
     for (; q + w.S < q1; q += 2 * w.S) {
@@ -935,7 +970,7 @@ __device__ void spmm_row_warp(const DevProblem& P, const T* Wm, int ld, int j, c
     // 32 entries a round: lane l forms the weight of entry l once (FP64, whose instructions take 16
     // clocks of the SM each whatever the lanes do: with every sub-team forming its own, the
     // weights of 8 entries cost as much as those of 32 here), then sub-team s takes the entries
-    // s, s + S, ..., their rows all in flight
+    // s, s + S, ...
     const int lane = threadIdx.x & 31;
     const int q1 = P.A_rp[j + 1];
     __syncwarp();
@@ -951,22 +986,10 @@ __device__ void spmm_row_warp(const DevProblem& P, const T* Wm, int ld, int j, c
         c = from_double<T>(x * to_double(av[q]));
       }
       const int rounds = min(32, q1 - q0);
-      for (int s0 = 0; s0 < rounds; s0 += 4 * w.S) {
-        Frag<T> Wk[4];
-        T ck[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int src = s0 + u * w.S + w.sub;          // < 32 when it is one of the entries
-          const int k = __shfl_sync(0xffffffffu, col, src & 31);
-          ck[u] = __shfl_sync(0xffffffffu, c, src & 31);
-          Team tw = t;
-          tw.nc = src < rounds ? t.nc : 0;
-          frag_load(Wk[u], Wm, k, ld, tw);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (s0 + u * w.S + w.sub < rounds) frag_axpy(acc, ck[u], Wk[u]);
-      }
+      int s0 = 0;
+      for (; rounds - s0 > w.S; s0 += H * w.S)
+        spmm_entries<T, H>(Wm, ld, s0, rounds, col, c, w, acc);
+      if (s0 < rounds) spmm_entries<T, 1>(Wm, ld, s0, rounds, col, c, w, acc);
     }
   }
   frag_warp_combine(acc, t.G);

@@ -54,6 +54,8 @@ inline int default_ctas(const SolveSize& p) {
 // is mostly past the row's end, and without it two CTAs of the FP64 kernel fit an SM where one does
 // (r = 9, one / two entries a round: n = 20,000 with 6 entries a row FP64 96 / 119 us, FP32 16.5 / 18.6;
 // n = 3,000 with 133 entries FP64 84 / 69).
+// The FP32 product's sub-teams then form their own entries' weights, for longer rows the warp
+// forms 32 at once (r = 9: 6 entries a row 13.3 / 22.1 us; 200 entries a row 41.6 / 31).
 inline bool short_rows(int64_t n, int64_t entries, int lanes) {
   return entries <= n * (32 / (lanes < 32 ? lanes : 32));
 }

@@ -78,24 +78,31 @@ __global__ void op_sddmm_kernel(DevProblem P, int ld, const T* U, const T* V, do
   }
 }
 
+// Diagonal constraints: one team per row.  A kernel of its own for its registers, as the Hessian's below
+// (FP32, 2^20 rows of r = 20: 161 us beside the other form, 128 alone)
 template <typename T>
+__global__ void op_spmm_diag_kernel(DevProblem P, int ld, const double* w, double gamma, const T* V,
+                                    T* out) {
+  const Team t = make_team(ld, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  for (int j = t.id; j < P.n; j += t.count) {
+    Frag<T> o;
+    spmm_row<T>(P, V, ld, j, w, nullptr, 0.0, 1.0, 0.0, (T)gamma, t, o);
+    frag_store(o, out, j, ld, t);
+  }
+}
+
+// FP32 with the warp's weights: two rows in flight per sub-team (H = 2) leave 48 registers, five CTAs per SM,
+// four take 72, three CTAs; four where the rows do not fill the five (r = 20, 200 entries a row, two / four:
+// n = 10,000 34.4 / 39.1 us, n = 6,400 31.0 / 26.8) and sub-teams have four of 32 entries
+template <typename T, bool OWN, int H>
 __global__ void op_spmm_kernel(DevProblem P, int ld, const double* w, double gamma, const T* V,
                                T* out) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-  if (P.a_diag_only) {
-    const Team t = make_team(ld, tid, nt);
-    for (int j = t.id; j < P.n; j += t.count) {
-      Frag<T> o;
-      spmm_row<T>(P, V, ld, j, w, nullptr, 0.0, 1.0, 0.0, (T)gamma, t, o);
-      frag_store(o, out, j, ld, t);
-    }
-  } else {
-    const WarpRow wr = make_warp_row(ld, tid, nt);
-    for (int j = wr.warp; j < P.n; j += wr.nwarps) {
-      Frag<T> o;
-      spmm_row_warp<T>(P, V, ld, j, w, nullptr, 0.0, 1.0, 0.0, (T)gamma, wr, o);
-      if (wr.sub == 0) frag_store(o, out, j, ld, wr.st);
-    }
+  const WarpRow wr =
+      make_warp_row(ld, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  for (int j = wr.warp; j < P.n; j += wr.nwarps) {
+    Frag<T> o;
+    spmm_row_warp<T, OWN, H>(P, V, ld, j, w, nullptr, 0.0, 1.0, 0.0, (T)gamma, wr, o);
+    if (wr.sub == 0) frag_store(o, out, j, ld, wr.st);
   }
 }
 
@@ -508,10 +515,18 @@ struct HessianF64Diag {
   template <>                                                                                  \
   cudaError_t Launch<T>::op_spmm(const DevProblem& P, int ld, const double* w, double gamma,   \
                                  const T* V, T* out, int grid, cudaStream_t s) {               \
-    if constexpr (sizeof(T) == 8) {                                                            \
-      if (P.a_diag_only) return launch_units<SpmmF64Diag>(ld, P.n, grid, s, P, ld, w, gamma, V, out); \
+    if (!P.a_diag_only) {                                                                      \
+      if (sizeof(T) == 8 || short_rows(P.n, P.a_nnz, team_size_for(ld)))                       \
+        op_spmm_kernel<T, true, 2><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);              \
+      else if (team_size_for(ld) >= 4 && P.n < 6 * grid)                                       \
+        op_spmm_kernel<T, sizeof(T) == 8, 4><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);    \
+      else                                                                                     \
+        op_spmm_kernel<T, sizeof(T) == 8, 2><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);    \
+    } else if constexpr (sizeof(T) == 8) {                                                     \
+      return launch_units<SpmmF64Diag>(ld, P.n, grid, s, P, ld, w, gamma, V, out);             \
+    } else {                                                                                   \
+      op_spmm_diag_kernel<T><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);                    \
     }                                                                                          \
-    op_spmm_kernel<T><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);                           \
     return cudaGetLastError();                                                                 \
   }                                                                                            \
   template <>                                                                                  \

@@ -26,7 +26,7 @@ def _instance(n, per_row, rng):
 
 @pytest.mark.parametrize("prec", [L.LORADS_PREC_FP64, L.LORADS_PREC_MIXED])
 @pytest.mark.parametrize("r", [4, 9, 16, 20, 40, 100])
-@pytest.mark.parametrize("n,per_row", [(400, 3), (150, 30), (201, 90)])
+@pytest.mark.parametrize("n,per_row", [(400, 3), (150, 30), (201, 90), (7400, 40)])
 def test_rows_of_uneven_lengths(cuda, prec, r, n, per_row):
     torch = cuda
     rng = np.random.default_rng(r + n)
