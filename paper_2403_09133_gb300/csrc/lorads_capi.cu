@@ -1287,7 +1287,7 @@ static int op_grid(const lorads_problem* p) {
     cudaGetLastError();
     sms = 1;
   }
-  return sms * 8;
+  return sms * OP_CTAS_PER_SM;
 }
 
 int lorads_op_sddmm(lorads_problem* p, int32_t prec, int32_t r, int32_t ld, const void* U,

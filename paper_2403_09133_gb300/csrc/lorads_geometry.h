@@ -60,4 +60,37 @@ inline bool short_rows(int64_t n, int64_t entries, int lanes) {
   return entries <= n * (32 / (lanes < 32 ? lanes : 32));
 }
 
+constexpr int OP_CTAS_PER_SM = 8;   // CTAs of an operator call's launch, per SM
+
+// FP64 operators: a row of ld doubles (ld <= 256) is ld / 2 units of 16 bytes, dealt to G lanes, at most
+// 8 units each.
+enum UnitWork { UNIT_SDDMM_DIAG, UNIT_SDDMM, UNIT_HESSIAN, UNIT_SPMM };
+inline int unit_count(int ld, int G) { return (ld / 2 + G - 1) / G; }
+
+// G: the fewest lanes, which issue the fewest FP64 instructions, widened up to 8 while the rows leave
+// SMs idle and latency counts instead.  How many lanes per SM are too few grows with the units that a
+// lane handles, one after the other; the product with C handles them once per entry of the row.
+// Measured at 1,000 to 80,000 rows, r = 9, 20, 32, 48, 2 / 4 / 8 lanes (us):
+//   sampled, on the diagonal   r = 9, n = 30,000  3.26 4.36 6.52     r = 32, n = 10,000  4.10 3.52 3.86
+//   sampled, off the diagonal  r = 9, n = 30,000  4.07 5.41 8.62     r = 32, n = 10,000  6.04 4.60 4.65
+//   Hessian                    r = 9, n = 30,000  5.24 7.16 9.73     r = 32, n = 20,000  10.6 8.47 8.92
+//   product, 7 entries a row   r = 9, n = 10,000  11.5 10.1 9.19     r = 20, n = 30,000  25.0 26.0 27.8
+// The product with 6 to 8 units per lane, whose sums take most registers, is widened further (degree 7,
+// wider / not: r = 48, 6 units, n = 40,000 50.7 / 60.1, n = 400,000 473 / 470; r = 32, 8 units, 41.6 / 53.6 and
+// 318 / 367).
+inline int unit_lanes(UnitWork work, int ld, long long rows, int sms) {
+  int G = 2;
+  while (unit_count(ld, G) > 8 || (work == UNIT_SPMM && G < 8 && unit_count(ld, G) == 8)) G <<= 1;
+  while (G < 8 && 2 * G <= ld / 2) {
+    const int N = unit_count(ld, G);
+    const int few = work == UNIT_SPMM         ? (N > 5 ? 3072 : 512)
+                    : work == UNIT_SDDMM_DIAG ? 26 * N
+                    : work == UNIT_SDDMM      ? 52 * N
+                                              : 36 * N;
+    if (rows * G >= (long long)sms * few) break;
+    G <<= 1;
+  }
+  return G;
+}
+
 }  // namespace lorads

@@ -455,28 +455,20 @@ struct Launch {
 LORADS_DECLARE_LAUNCH(double)
 LORADS_DECLARE_LAUNCH(float)
 
-// lanes per row and units per lane of the FP64 operators (ld <= 256): the fewest lanes that leave at
-// most 8 units each, which issue the fewest FP64 instructions; up to 8 where
-// the rows alone would not fill the SMs with 16 warps and latency counts instead (2 lanes per row
-// took 29 us for a product that 8 lanes form in 14)
-inline int unit_lanes(int ld, long long rows) {
-  int G = 2;
-  while ((ld / 2 + G - 1) / G > 8) G <<= 1;
-  while (G < 8 && 2 * G <= ld / 2 && rows * G < 152LL * 512) G <<= 1;
-  return G;
-}
+// (lanes per row: unit_lanes; work: the operator's cost)
 template <template <int> class K, class... A>
-inline cudaError_t launch_units(int ld, long long rows, A... args) {
-  const int G = unit_lanes(ld, rows);
-  switch ((ld / 2 + G - 1) / G) {
-    case 1: K<1>::go(G, args...); break;
-    case 2: K<2>::go(G, args...); break;
-    case 3: K<3>::go(G, args...); break;
-    case 4: K<4>::go(G, args...); break;
-    case 5: K<5>::go(G, args...); break;
-    case 6: K<6>::go(G, args...); break;
-    case 7: K<7>::go(G, args...); break;
-    default: K<8>::go(G, args...); break;
+inline cudaError_t launch_units(UnitWork work, int ld, long long rows, int grid, cudaStream_t s,
+                                const A&... args) {
+  const int G = unit_lanes(work, ld, rows, grid / OP_CTAS_PER_SM);
+  switch (unit_count(ld, G)) {
+    case 1: K<1>::go(G, grid, s, args...); break;
+    case 2: K<2>::go(G, grid, s, args...); break;
+    case 3: K<3>::go(G, grid, s, args...); break;
+    case 4: K<4>::go(G, grid, s, args...); break;
+    case 5: K<5>::go(G, grid, s, args...); break;
+    case 6: K<6>::go(G, grid, s, args...); break;
+    case 7: K<7>::go(G, grid, s, args...); break;
+    default: K<8>::go(G, grid, s, args...); break;
   }
   return cudaGetLastError();
 }
@@ -507,7 +499,8 @@ struct HessianF64Diag {
   template <>                                                                                  \
   cudaError_t Launch<T>::op_sddmm(const DevProblem& P, int ld, const T* U, const T* V,         \
                                   double* q, int grid, cudaStream_t s) {                       \
-    if constexpr (sizeof(T) == 8) return launch_units<SddmmF64>(ld, P.m, grid, s, P, ld, U, V, q);  \
+    if constexpr (sizeof(T) == 8) return launch_units<SddmmF64>(P.a_diag_only ? UNIT_SDDMM_DIAG : UNIT_SDDMM, \
+                                                              ld, P.m, grid, s, P, ld, U, V, q); \
     else if (P.a_multi) op_sddmm_kernel<T, true><<<grid, 256, 0, s>>>(P, ld, U, V, q);         \
     else op_sddmm_kernel<T, false><<<grid, 256, 0, s>>>(P, ld, U, V, q);                       \
     return cudaGetLastError();                                                                 \
@@ -518,12 +511,12 @@ struct HessianF64Diag {
     if (!P.a_diag_only) {                                                                      \
       if (sizeof(T) == 8 || short_rows(P.n, P.a_nnz, team_size_for(ld)))                       \
         op_spmm_kernel<T, true, 2><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);              \
-      else if (team_size_for(ld) >= 4 && P.n < 6 * grid)                                       \
+      else if (team_size_for(ld) >= 4 && P.n < 48 * (grid / OP_CTAS_PER_SM))                                      \
         op_spmm_kernel<T, sizeof(T) == 8, 4><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);    \
       else                                                                                     \
         op_spmm_kernel<T, sizeof(T) == 8, 2><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);    \
     } else if constexpr (sizeof(T) == 8) {                                                     \
-      return launch_units<SpmmF64Diag>(ld, P.n, grid, s, P, ld, w, gamma, V, out);             \
+      return launch_units<SpmmF64Diag>(UNIT_SPMM, ld, P.n, grid, s, P, ld, w, gamma, V, out);  \
     } else {                                                                                   \
       op_spmm_diag_kernel<T><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);                    \
     }                                                                                          \
@@ -543,7 +536,8 @@ struct HessianF64Diag {
       else                                                                                     \
         op_hessian_kernel<T, 2><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, out);     \
     } else if constexpr (sizeof(T) == 8) {                                                     \
-      return launch_units<HessianF64Diag>(ld, P.n, grid, s, P, ld, rho, gamma, V, Pm, out);         \
+      return launch_units<HessianF64Diag>(UNIT_HESSIAN, ld, P.n, grid, s, P, ld, rho, gamma, V,    \
+                                          Pm, out);                                            \
     } else {                                                                                   \
       op_hessian_diag_kernel<T><<<grid, 256, 0, s>>>(P, ld, (T)rho, (T)gamma, V, Pm, out);     \
     }                                                                                          \

@@ -18,6 +18,12 @@ int main(int argc, char** argv) {
     std::printf("%d\n", (int)lorads::short_rows(atol(argv[2]), atol(argv[3]), atoi(argv[4])));
     return 0;
   }
+  if (argc == 6 && argv[1][0] == 'u') {
+    const int G = lorads::unit_lanes((lorads::UnitWork)atoi(argv[2]), atoi(argv[3]), atol(argv[4]),
+                                     atoi(argv[5]));
+    std::printf("%d\n%d\n", G, lorads::unit_count(atoi(argv[3]), G));
+    return 0;
+  }
   for (int i = 1; i + 5 < argc; i += 6) {
     lorads::SolveSize s{};
     s.n = atol(argv[i]);
@@ -90,3 +96,29 @@ def test_short_rows(ctas):
         for n in (1, 20000):
             assert ctas.call("s", n, n * S, lanes) == [1]
             assert ctas.call("s", n, n * S + 1, lanes) == [0]
+
+
+def test_unit_lanes(ctas):
+    """FP64 operators: at most 8 units per lane and a lane for every unit at most; two lanes with many
+    rows, eight with few; no widening where it was measured to lose."""
+    SDDMM_DIAG, SDDMM, HESSIAN, SPMM = range(4)
+
+    def lanes(work, ld, rows):
+        G, N = ctas.call("u", work, ld, rows, 152)
+        assert G in (2, 4, 8, 16) and N <= 8 and (N - 1) * G < ld // 2 <= N * G
+        return G
+
+    for work in range(4):
+        for ld in range(4, 257, 4):
+            least = next(G for G in (2, 4, 8, 16) if G * 8 >= ld // 2)
+            if work == SPMM and least < 8 and -(-(ld // 2) // least) == 8:
+                least *= 2
+            assert lanes(work, ld, 10 ** 7) == least
+            few = lanes(work, ld, 100)
+            assert few == max(least, min(8, 1 << (ld // 2).bit_length() - 1))
+            sizes = [lanes(work, ld, rows) for rows in (100, 1000, 10 ** 4, 10 ** 5, 10 ** 6)]
+            assert sizes == sorted(sizes, reverse=True)
+    assert lanes(SDDMM_DIAG, 12, 30000) == 2 and lanes(SDDMM, 12, 30000) == 2
+    assert lanes(HESSIAN, 12, 30000) == 2 and lanes(HESSIAN, 32, 20000) == 4
+    assert lanes(SDDMM_DIAG, 32, 10000) == 4 and lanes(SPMM, 48, 10000) == 8
+    assert lanes(SPMM, 32, 10 ** 6) == 4 and lanes(SPMM, 48, 80000) == 8 and lanes(SPMM, 20, 80000) == 2
