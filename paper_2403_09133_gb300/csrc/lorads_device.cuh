@@ -407,8 +407,8 @@ __device__ inline void block_reduce(double* v, int k, double* red /* smem [33*MA
 // reduce_pair sums two values given in warp_sums_pair's form and calls f(sum 0, sum 1) in thread 0
 // of every CTA before the CTA goes on: f evaluates the scalars that follow from the sums (FP64
 // divides issue at 1/64 of the FP32 rate here, so one thread per CTA does it) and leaves them in
-// the scratch row.  reduce_each(v, k, f) calls f(i, sum i) for each value in one thread of the
-// CTA.  EXCHANGE tells whether the scope's CTAs also read one another's memory writes after it;
+// the scratch row.  reduce_each<K>(v, f) calls f(i, sum i) for each of K values in one thread of
+// the CTA.  EXCHANGE tells whether the scope's CTAs also read one another's memory writes after it;
 // without, a reduction orders nothing but its sums.
 struct BlockScope {
   double* red;
@@ -419,7 +419,12 @@ struct BlockScope {
     __syncthreads();
     return true;
   }
-  __device__ bool reduce(double* v, int k) {
+  template <int K>
+  __device__ __forceinline__ bool reduce(double* v) {
+    static_assert(K >= 1 && K < MAXRED, "a row of the shared array holds a reduction's values");
+    return reduce_any(v, K);
+  }
+  __device__ bool reduce_any(double* v, int k) {
     block_reduce(v, k, red);
     return true;
   }
@@ -439,8 +444,10 @@ struct BlockScope {
     __syncthreads();
     return true;
   }
-  template <class F>
-  __device__ __forceinline__ bool reduce_each(const double* v, int k, F f) {
+  template <int K, class F>
+  __device__ __forceinline__ bool reduce_each(const double* v, F f) {
+    static_assert(K >= 1 && K < MAXRED, "a row of the shared array holds a reduction's values");
+    constexpr int k = K;
     const int nw = (blockDim.x + 31) >> 5;
     warp_sums(v, k, red);
     __syncthreads();
@@ -592,8 +599,13 @@ struct GridScope {
   }
 
   // f(i, sum i) in lane 0 of the warp that finishes value i
+  template <int K, class F>
+  __device__ __forceinline__ bool reduce_each(const double* v, F f) {
+    static_assert(K >= 1 && K <= SLOT_VALUES, "a set of slots holds a reduction's values");
+    return each_any(v, K, f);
+  }
   template <class F>
-  __device__ __forceinline__ bool reduce_each(const double* v, int k, F f) {
+  __device__ __forceinline__ bool each_any(const double* v, int k, F f) {
     const int nw = (blockDim.x + 31) >> 5;
     warp_sums(v, k, red);
     const unsigned bar = ++gen;
@@ -605,9 +617,14 @@ struct GridScope {
     __syncthreads();
     return !failed();
   }
-  __device__ bool reduce(double* v, int k) {
+  template <int K>
+  __device__ __forceinline__ bool reduce(double* v) {
+    static_assert(K >= 1 && K <= SLOT_VALUES, "a set of slots holds a reduction's values");
+    return reduce_any(v, K);
+  }
+  __device__ bool reduce_any(double* v, int k) {
     double* out = red + 32 * MAXRED;
-    const bool ok = reduce_each(v, k, [out](int i, double s) { out[i] = s; });
+    const bool ok = each_any(v, k, [out](int i, double s) { out[i] = s; });
     for (int i = 0; i < k; ++i) v[i] = out[i];
     return ok;
   }

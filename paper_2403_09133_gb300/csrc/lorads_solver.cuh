@@ -358,7 +358,7 @@ struct Solver {
         }
       }
     }
-    if (!sc.reduce(v, 1)) return false;
+    if (!sc.template reduce<1>(v)) return false;
     e2 = v[0];
     return true;
   }
@@ -404,7 +404,7 @@ struct Solver {
         if (wr.sub == 0 && wr.st.lead) v[0] += d;
       }
     }
-    if (!sc.reduce(v, 1)) return false;
+    if (!sc.template reduce<1>(v)) return false;
     g2 = v[0];
     return true;
   }
@@ -438,7 +438,7 @@ struct Solver {
         const double d = frag_dot(g, g, tm);
         if (tm.lead) v[0] -= d;
       }
-      if (!sc.reduce(v, 1)) return false;
+      if (!sc.template reduce<1>(v)) return false;
       dg = v[0];
       return true;
     }
@@ -464,7 +464,7 @@ struct Solver {
         const double d = frag_dot(s, q, tm);
         if (tm.lead) v[0] += d;
       }
-      if (!sc.reduce(v, 1)) return false;
+      if (!sc.template reduce<1>(v)) return false;
       alpha[i] = hrho[slot] * v[0];
     }
     // loop 2: oldest -> newest, starting from H0 (q - alpha_last y_last)
@@ -497,7 +497,7 @@ struct Solver {
         const double d = frag_dot(y, q, tm);
         if (tm.lead) v[0] += d;
       }
-      if (!sc.reduce(v, 1)) return false;
+      if (!sc.template reduce<1>(v)) return false;
       beta_prev = hrho[slot] * v[0];
     }
     {
@@ -520,7 +520,7 @@ struct Solver {
         const double d = frag_dot(q, g, tm);
         if (tm.lead) v[0] += d;
       }
-      if (!sc.reduce(v, 1)) return false;
+      if (!sc.template reduce<1>(v)) return false;
       dg = v[0];
     }
     return true;
@@ -600,7 +600,7 @@ struct Solver {
         if (tmc.lead) accumulate(i, e1, e2);
       }
     }
-    if (!sc.reduce(v, 9)) return false;
+    if (!sc.template reduce<9>(v)) return false;
     a[0] = v[7] + v[0] + sigma * v[2];
     a[1] = v[8] + v[1] + 0.5 * sigma * (v[4] + 2.0 * v[3]);
     a[2] = sigma * v[5];
@@ -655,7 +655,7 @@ struct Solver {
         v[1] += b;
       }
     }
-    if (!sc.reduce(v, 2)) return false;
+    if (!sc.template reduce<2>(v)) return false;
     sy = v[0];
     yy = v[1];
     return true;
@@ -868,7 +868,7 @@ struct Solver {
         v[1] += a2;
       }
     }
-    if (!sc.reduce(v, 2)) return false;
+    if (!sc.template reduce<2>(v)) return false;
     ++hess;
     const T rho_t = (T)rho, gamma_t = (T)gamma;
     int it = 0;
@@ -898,7 +898,7 @@ struct Solver {
         const T d = team_sum(frag_dot_local(Pj, Hj), st);
         if (wr.sub == 0 && st.lead) w[0] += to_double(d);
       }
-      if (!sc.reduce_each(w, 1, [this, own](int, double pHp) {
+      if (!sc.template reduce_each<1>(w, [this, own](int, double pHp) {
             if (!(pHp > 0.0)) cg_leave(pHp == pHp ? 1 : 2, 0.0, 0.0);
             else cg_leave(0, own[0] / pHp, 0.0);
           }))
@@ -924,7 +924,7 @@ struct Solver {
         const double d = frag_dot(Rd, Rd, tm);
         if (tm.lead) z[0] += d;
       }
-      if (!sc.reduce_each(z, 1, [this, own](int, double rr_new) {
+      if (!sc.template reduce_each<1>(z, [this, own](int, double rr_new) {
             // stop on the new residual; beta otherwise (a NaN goes on, as p.Hp then shows it)
             if (sqrt(rr_new) <= own[1]) {
               cg_leave(1, 0.0, 0.0);
@@ -1156,7 +1156,7 @@ struct Solver {
       v[2] = dv[0];
       v[3] = dv[1];
       if (sc.is_leader()) v[4] = (double)(globaltimer_ns() - t_start);
-      if (!sc.reduce(v, 5)) return false;
+      if (!sc.template reduce<5>(v)) return false;
       admm_iters = k + 1;
       log_iter(k, rho, v[0], v[1], v[4]);
       double s3[3];
@@ -1316,7 +1316,7 @@ struct Solver {
       frag_store(mCW, A.CWn, j, ld, tm);
       local_r0_row(j, Wj, Wjt, mCW, c, c.lam, rho, gamma, tm, g3, dout);
     }
-    if (!sc.reduce(g3, 3)) return false;
+    if (!sc.template reduce<3>(g3)) return false;
     ++hess;
     return true;
   }
@@ -1569,7 +1569,7 @@ struct Solver {
         const double qU = local_r0_row(j, Xj, Xt, mCX, c, c.lam, rho, gamma, tm, g3);
         if (c.i >= 0 && tm.lead) A.e[c.i] = qU;  // a ||U_j^{k+1}||^2 for the output residual
       }
-      if (!sc.reduce(g3, 3)) return false;
+      if (!sc.template reduce<3>(g3)) return false;
       ++hess;
       // V-step: CG on eq. linV (W = U^{k+1})
       if (!cg_local_loop(A.Ut, rho, gamma, g3, it)) return false;
@@ -1630,7 +1630,7 @@ struct Solver {
         }
       }
       if (sc.is_leader()) v[4] = (double)(globaltimer_ns() - t_start);
-      if (!sc.reduce(v, 8)) return false;
+      if (!sc.template reduce<8>(v)) return false;
       ++hess;
       g3[0] = v[5];
       g3[1] = v[6];
@@ -1764,7 +1764,7 @@ struct Solver {
         }
       }
       if (sc.is_leader()) v[4] = (double)(globaltimer_ns() - t_start);
-      if (!sc.reduce(v, 5)) return false;
+      if (!sc.template reduce<5>(v)) return false;
       ++hess;
       admm_iters = k + 1;
       log_iter(k, rho, v[0], v[1], v[4]);
@@ -1868,7 +1868,7 @@ struct Solver {
       }
     }
     if (sc.is_leader()) v[3] = (double)(globaltimer_ns() - t_start);
-    return sc.reduce(v, 4);
+    return sc.template reduce<4>(v);
   }
 
   // One pass of the truncated CG for row j: with the scalars (a, b) of the step, p = r + b p,
@@ -1996,7 +1996,7 @@ struct Solver {
         g3[1] += d2;
       }
     }
-    if (!sc.reduce(g3, 2)) return false;
+    if (!sc.template reduce<2>(g3)) return false;
     const double eta = fmin(0.5, sqrt(sqrt(g2)));
     const double target2 = eta * eta * g2;
     const double dl2 = delta * delta;
@@ -2148,7 +2148,7 @@ struct Solver {
         v[1] += a2;
       }
     }
-    if (!sc.reduce(v, 2)) return false;
+    if (!sc.template reduce<2>(v)) return false;
     pred = -(v[0] + 0.5 * v[1]);
     return true;
   }
@@ -2178,7 +2178,7 @@ struct Solver {
         for (int e = 0; e < CHUNK; ++e) Uj.v[k][e] *= sc2;
       frag_store(Uj, A.V, j, ld, tm);
     }
-    if (!sc.reduce(v, 1)) return false;
+    if (!sc.template reduce<1>(v)) return false;
     if (want_slope) slope = v[0];
     return true;
   }
@@ -2195,7 +2195,7 @@ struct Solver {
       const double o = -frag_dot(Wj, mCW, tm);
       if (tm.lead) v[0] += o;
     }
-    if (!sc.reduce(v, 1)) return false;
+    if (!sc.template reduce<1>(v)) return false;
     f = v[0];
     return true;
   }
@@ -2306,7 +2306,7 @@ struct Solver {
       const double d = frag_dot(Uj, Uj, tm);
       if (tm.lead) v[0] += d;
     }
-    if (!sc.reduce(v, 1)) return false;
+    if (!sc.template reduce<1>(v)) return false;
     u2 = v[0];
     return true;
   }
@@ -2413,7 +2413,7 @@ struct Solver {
       }
     }
     for (int i = sc.tid(); i < m; i += sc.nthreads()) v[1] += P.b[i] * A.lam[i];
-    if (!sc.reduce(v, 4)) return false;
+    if (!sc.template reduce<4>(v)) return false;
     uh_norm2 = v[2];
     last_rd2 = v[3];
     const double pobj = v[0], dobj = -v[1];
@@ -2508,7 +2508,7 @@ struct Solver {
           for (int k = 0; k < NC; ++k) v[k] = (k == warp && below < Lc) ? 1.0 : 0.0;
         }
       }
-      if (!sc.reduce(v, NC)) return false;
+      if (!sc.template reduce<NC>(v)) return false;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         if (Ls[c] <= 0) continue;
@@ -2599,7 +2599,7 @@ struct Solver {
         Qp[(long long)j * NC + c] = 0.0;
         v[c] += x * x;
       }
-    if (!sc.reduce(v, NC)) return false;
+    if (!sc.template reduce<NC>(v)) return false;
     double qs[NC], qps[NC], bp[NC], qs0[NC];
     int len[NC];
 #pragma unroll
@@ -2632,7 +2632,7 @@ struct Solver {
           a[c] += qs[c] * Q[o + c] * w;
         }
       }
-      if (!sc.reduce(a, NC)) return false;
+      if (!sc.template reduce<NC>(a)) return false;
       // W -= alpha_k q_k;  beta_k = ||W||
       double b2[NC] = {0.0, 0.0, 0.0, 0.0};
       for (int j = sc.tid(); j < n; j += sc.nthreads()) {
@@ -2647,7 +2647,7 @@ struct Solver {
       // beta_k = ||W||, the scale of q_{k+1} and the column's length, for each column in the thread
       // that holds its sum; every thread reads them from the scratch row
       double* const nxt = sc.scratch();     // 1/beta, beta, length of the four columns
-      if (!sc.reduce_each(b2, NC, [&](int c, double w2) {
+      if (!sc.template reduce_each<NC>(b2, [&](int c, double w2) {
             double ac = a[0], bc = bp[0];
             int lc = len[0];
 #pragma unroll
@@ -2836,7 +2836,7 @@ struct Solver {
     }
     double z2[1] = {0.0};
     for (int j = sc.tid(); j < n; j += sc.nthreads()) z2[0] += zv[j] * zv[j];
-    if (!sc.reduce(z2, 1)) return false;
+    if (!sc.template reduce<1>(z2)) return false;
     *zn2 = z2[0];
     return true;
   }
@@ -2945,7 +2945,7 @@ struct Solver {
         if (tmc.lead) add(i, q, qs);
       }
     }
-    if (!sc.reduce(v, 5)) return false;
+    if (!sc.template reduce<5>(v)) return false;
     for (int i = 0; i < 5; ++i) res[i] = v[i];
     return true;
   }
