@@ -574,19 +574,30 @@ struct GridScope {
   }
   __device__ bool failed() const { return red[32 * MAXRED + MAXRED - 1] != 0.0; }
 
-  // One warp: stores the CTA's sum x of value i (the same in every lane below 16) and returns the
-  // sum over the scope in every lane.  `bar` is the barrier's number.
-  template <bool EXCHANGE>
-  __device__ __forceinline__ double exchange(double x, int i, unsigned bar) {
+  // One warp: stores the CTA's sum x of value i (the same in every lane below 16) for barrier `bar`
+  __device__ __forceinline__ void put(double x, int i, unsigned bar) {
     const int lane = threadIdx.x & 31, c = count(), me = (int)blockIdx.x - first;
     const size_t copy = (size_t)2 * SLOT_VALUES * c;
     Slot* set = slots + ((size_t)(bar & 1u) * SLOT_VALUES + i) * c;
-    if (EXCHANGE) fence_release_gpu();
     if (lane < reps) st_slot(set + lane * copy + me, x, bar);
+  }
+  // One warp: the sum of value i over the scope, in every lane
+  __device__ __forceinline__ double take(int i, unsigned bar) {
+    const int c = count(), me = (int)blockIdx.x - first;
+    const size_t copy = (size_t)2 * SLOT_VALUES * c;
+    const Slot* set = slots + ((size_t)(bar & 1u) * SLOT_VALUES + i) * c;
     bool ok = true;
     const double s = poll_slots(set + (me % reps) * copy, c, bar, &ctl->error, spin_limit, ok);
-    if (EXCHANGE) fence_acquire_gpu();
     if (!ok) red[32 * MAXRED + MAXRED - 1] = 1.0;
+    return s;
+  }
+  // both, for a warp with one value
+  template <bool EXCHANGE>
+  __device__ __forceinline__ double exchange(double x, int i, unsigned bar) {
+    if (EXCHANGE) fence_release_gpu();
+    put(x, i, bar);
+    const double s = take(i, bar);
+    if (EXCHANGE) fence_acquire_gpu();
     return s;
   }
 
@@ -610,8 +621,14 @@ struct GridScope {
     warp_sums(v, k, red);
     const unsigned bar = ++gen;
     __syncthreads();
-    for (int i = threadIdx.x >> 5; i < k; i += nw) {
-      const double s = exchange<true>(block_sum(i, red), i, bar);
+    // a warp stores all of its values before it waits for any: one trip through L2, and not three, for
+    // the line search's 9 values in CTAs of 4 warps
+    const int warp = threadIdx.x >> 5;
+    if (warp < k) fence_release_gpu();
+    for (int i = warp; i < k; i += nw) put(block_sum(i, red), i, bar);
+    for (int i = warp; i < k; i += nw) {
+      const double s = take(i, bar);
+      fence_acquire_gpu();
       if ((threadIdx.x & 31) == 0) f(i, s);
     }
     __syncthreads();
