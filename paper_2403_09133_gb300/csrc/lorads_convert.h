@@ -4,7 +4,8 @@
 // clocks here (1/64 of the FP32 rate), and the solver's mixed form converts three or four values
 // per element of every row pass.  These take 6 and 12 integer instructions, which the four
 // schedulers of an SM issue in parallel.  The results are those of the casts for every input: the
-// common cases (normal numbers and zeros) are formed here, the others are left to the cast.
+// common cases (normal numbers and zeros) are formed here, the others are left to the cast.  (Tested on
+// host and device for every float and at every boundary between two normal floats.)
 #pragma once
 #include <stdint.h>
 #include <string.h>

@@ -19,8 +19,8 @@
 //     A shuffle that names only its team's lanes splits the warp: one 8-element dot product with
 //     its team sum took 478 clocks in teams of 2 and 552 in teams of 4 (9 warps per SM), 126 and
 //     169 with the whole warp named.
-//   * Reductions are deterministic: fixed shuffle trees inside warps, warps summed in order,
-//     CTAs summed in order by the last CTA to arrive at the grid barrier.
+//   * Reductions are deterministic: fixed shuffle trees inside warps and over a CTA's warps; over
+//     CTAs every CTA adds the same sums in the same order (GridScope).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -242,9 +242,11 @@ __device__ __forceinline__ T frag_dot_local(const Frag<T>& a, const Frag<T>& b) 
 }
 
 // Sum over the lanes of each team, called by whole warps.  The lanes arrive here from loads that
-// only some of them make (a row's last chunks) and converge before they exchange: without that
-// the one-CTA FP64 kernel, depending on how it was compiled, exchanged across lanes that had not
-// met (matrix completion, r = 9, ld = 12: lane 1 of a team has no second chunk).
+// only some of them make (a row's last chunks: r = 9, ld = 12, lane 1 of a team has no second one) and
+// converge before they exchange.  Builds of the one-CTA FP64 kernel that named only the team's lanes
+// and did not converge them diverged on matrix completion, depending on how they were compiled, and
+// became exact with a convergence here and nothing else changed.  The shuffle waits for the lanes
+// it names by itself, so why that mattered is not known; it has not been seen since.
 template <typename T>
 __device__ __forceinline__ T team_sum(T x, const Team& t) {
   __syncwarp();
@@ -622,7 +624,7 @@ struct GridScope {
     const unsigned bar = ++gen;
     __syncthreads();
     // a warp stores all of its values before it waits for any: one trip through L2, and not three, for
-    // the line search's 9 values in CTAs of 4 warps
+    // the line search's 9 values in CTAs of 4 warps (Phase I of ER n = 1,600 5.5 -> 5.2 ms)
     const int warp = threadIdx.x >> 5;
     if (warp < k) fence_release_gpu();
     for (int i = warp; i < k; i += nw) put(block_sum(i, red), i, bar);

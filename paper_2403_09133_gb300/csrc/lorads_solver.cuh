@@ -5,8 +5,9 @@
 // (Algorithm 1 with warm-started CG on eq. linU / eq. linV, dual step, penalty schedule)
 // and the output step U_hat = (U + V)/2 with its residuals.  It is written once against a
 // "scope": one CTA (BlockScope: small problems and batches, one CTA per problem) or the
-// whole grid of a cooperative launch (GridScope: one large problem).  Every scalar decision
-// is taken redundantly by all threads from reduced values, so control flow is uniform.
+// whole grid of a cooperative launch (GridScope: one large problem).  Every CTA takes the same
+// decisions from the same sums; scalars that need FP64 divisions or roots are evaluated by one thread
+// of the CTA and shared, the others by all threads, so control flow is uniform.
 //
 // Precision: T is the element type of the CG operators and vectors (double: plain FP64,
 // float: mixed form).  The masters U, V, lambda, the CG scalars alpha/beta, all residual
