@@ -708,7 +708,17 @@ struct Solver {
   // the bulk products on the FP64 masters, until r_P <= tol and r_D <= tol, where r_D of the
   // multiplier-updated pair is ||grad phi|| / (2 (1 + ||C||_F)) at the end of an inner solve.
   // alm_done tells whether the stopping rule was met (else max_outer ran out).
-  __device__ bool alm(double& sigma_io, bool refine, int max_outer) {
+  // In the mixed form a function of its own, as cg_solve: inlined, the general form's code took registers
+  // from Phase III's truncated CG (141^2 torus 298 ms, apart 284); in FP64 inlined (theta n = 2,000
+  // 2.08 ms per L-BFGS iteration, apart 2.24).
+  __device__ __forceinline__ bool alm(double& sigma_io, bool refine, int max_outer) {
+    if constexpr (sizeof(T) == 4) return alm_apart(sigma_io, refine, max_outer);
+    else return alm_body(sigma_io, refine, max_outer);
+  }
+  __device__ __noinline__ bool alm_apart(double& sigma_io, bool refine, int max_outer) {
+    return alm_body(sigma_io, refine, max_outer);
+  }
+  __device__ __forceinline__ bool alm_body(double& sigma_io, bool refine, int max_outer) {
     double sigma;
     if (!refine) {
       for (int i = sc.tid(); i < m; i += sc.nthreads()) A.lam[i] = 0.0;
@@ -806,8 +816,18 @@ struct Solver {
   // R_0 = G - H W with G = (A^T(rho b - lambda) - C) W + gamma W, computed in FP64:
   //   R_0j = sum_{entries} a (rho b_i - lambda_i - rho q_i) W_k - (C W)_j,
   //   q_i = <A_i, W W^T>  (the gamma terms cancel because X_0 = W).
-  __device__ bool cg_solve(const double* Wm, const T* Wt, double* Xm, T* Xt, double rho,
-                           double gamma, bool want_dv, double* dv) {
+  __device__ __forceinline__ bool cg_solve(const double* Wm, const T* Wt, double* Xm, T* Xt,
+                                           double rho, double gamma, bool want_dv, double* dv) {
+    if constexpr (sizeof(T) == 4) return cg_solve_apart(Wm, Wt, Xm, Xt, rho, gamma, want_dv, dv);
+    else return cg_solve_body(Wm, Wt, Xm, Xt, rho, gamma, want_dv, dv);
+  }
+  __device__ __noinline__ bool cg_solve_apart(const double* Wm, const T* Wt, double* Xm, T* Xt,
+                                              double rho, double gamma, bool want_dv, double* dv) {
+    return cg_solve_body(Wm, Wt, Xm, Xt, rho, gamma, want_dv, dv);
+  }
+  __device__ __forceinline__ bool cg_solve_body(const double* Wm, const T* Wt, double* Xm, T* Xt,
+                                                double rho, double gamma, bool want_dv,
+                                                double* dv) {
     double v[2] = {0.0, 0.0};
     // one warp per row (entries split across sub-teams): rows with many entries
     const WarpRow wr = make_warp_row(ld, sc.tid(), sc.nthreads(), prm.team_mult);
