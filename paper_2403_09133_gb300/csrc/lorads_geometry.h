@@ -75,7 +75,8 @@ inline int unit_count(int ld, int G) { return (ld / 2 + G - 1) / G; }
 //   sampled, off the diagonal  r = 9, n = 30,000  4.07 5.41 8.62     r = 32, n = 10,000  6.04 4.60 4.65
 //   Hessian                    r = 9, n = 30,000  5.24 7.16 9.73     r = 32, n = 20,000  10.6 8.47 8.92
 //   product, 7 entries a row   r = 9, n = 10,000  11.5 10.1 9.19     r = 20, n = 30,000  25.0 26.0 27.8
-// The product with 6 to 8 units per lane, whose sums take most registers, is widened further (degree 7,
+// The Hessian and the product with 6 to 8 units per lane, whose rows take most registers, are widened
+// further (Hessian r = 48, n = 10,000, 6 units 8.2, 3 units 7.3; product of degree 7,
 // wider / not: r = 48, 6 units, n = 40,000 50.7 / 60.1, n = 400,000 473 / 470; r = 32, 8 units, 41.6 / 53.6 and
 // 318 / 367).
 inline int unit_lanes(UnitWork work, int ld, long long rows, int sms) {
@@ -86,6 +87,7 @@ inline int unit_lanes(UnitWork work, int ld, long long rows, int sms) {
     const int few = work == UNIT_SPMM         ? (N > 5 ? 3072 : 512)
                     : work == UNIT_SDDMM_DIAG ? 26 * N
                     : work == UNIT_SDDMM      ? 52 * N
+                    : N > 5                   ? 512
                                               : 36 * N;
     if (rows * G >= (long long)sms * few) break;
     G <<= 1;

@@ -78,15 +78,43 @@ __global__ void op_sddmm_kernel(DevProblem P, int ld, const T* U, const T* V, do
   }
 }
 
-// Diagonal constraints: one team per row.  A kernel of its own for its registers, as the Hessian's below
-// (FP32, 2^20 rows of r = 20: 161 us beside the other form, 128 alone)
-template <typename T>
-__global__ void op_spmm_diag_kernel(DevProblem P, int ld, const double* w, double gamma, const T* V,
-                                    T* out) {
+// Diagonal constraints: one team per row, H of C's entries a round, their rows in flight together.  A
+// kernel of its own: beside the form below, which took 72 registers, 2^20 rows of r = 20 took 161 us (FP32),
+// here 89.  Few rows wait for their loads and take eight entries a round, many fill the SMs at four.
+template <typename T, int H>
+__global__ void __launch_bounds__(256, H == 8 ? 2 : 5)
+op_spmm_diag_kernel(DevProblem P, int ld, const double* w, double gamma, const T* V, T* out) {
   const Team t = make_team(ld, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  const T *ra = rowa<T>(P), *cv = cval<T>(P);
+  const T g = (T)gamma;
   for (int j = t.id; j < P.n; j += t.count) {
-    Frag<T> o;
-    spmm_row<T>(P, V, ld, j, w, nullptr, 0.0, 1.0, 0.0, (T)gamma, t, o);
+    // the row's own terms from the per-row arrays, asked for before C's entries: through A's rows they
+    // wait for four loads in a row after those
+    const int con = P.row_con[j];
+    const double wj = con >= 0 ? w[con] : 0.0;
+    const T a = ra[j];
+    Frag<T> Vj, o;
+    frag_load(Vj, V, j, ld, t);
+    frag_zero(o);
+    const int q1 = P.C_rp[j + 1];
+    for (int q = P.C_rp[j]; q < q1; q += H) {
+      Frag<T> W[H];
+      T c[H];
+#pragma unroll
+      for (int u = 0; u < H; ++u) {
+        // an entry past the row's end is neither read nor added
+        const bool on = q + u < q1;
+        Team tu = t;
+        tu.nc = on ? t.nc : 0;
+        c[u] = on ? cv[q + u] : T(0);
+        frag_load(W[u], V, on ? P.C_col[q + u] : j, ld, tu);
+      }
+#pragma unroll
+      for (int u = 0; u < H; ++u)
+        if (q + u < q1) frag_axpy(o, -c[u], W[u]);
+    }
+    if (con >= 0) frag_axpy(o, (T)(wj * (double)a), Vj);
+    if (g != T(0)) frag_axpy(o, g, Vj);
     frag_store(o, out, j, ld, t);
   }
 }
@@ -517,8 +545,10 @@ struct HessianF64Diag {
         op_spmm_kernel<T, sizeof(T) == 8, 2><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);    \
     } else if constexpr (sizeof(T) == 8) {                                                     \
       return launch_units<SpmmF64Diag>(UNIT_SPMM, ld, P.n, grid, s, P, ld, w, gamma, V, out);  \
+    } else if ((long long)P.n * team_size_for(ld) < 512LL * (grid / OP_CTAS_PER_SM)) {         \
+      op_spmm_diag_kernel<T, 8><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);                 \
     } else {                                                                                   \
-      op_spmm_diag_kernel<T><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);                    \
+      op_spmm_diag_kernel<T, 4><<<grid, 256, 0, s>>>(P, ld, w, gamma, V, out);                 \
     }                                                                                          \
     return cudaGetLastError();                                                                 \
   }                                                                                            \

@@ -120,5 +120,6 @@ def test_unit_lanes(ctas):
             assert sizes == sorted(sizes, reverse=True)
     assert lanes(SDDMM_DIAG, 12, 30000) == 2 and lanes(SDDMM, 12, 30000) == 2
     assert lanes(HESSIAN, 12, 30000) == 2 and lanes(HESSIAN, 32, 20000) == 4
+    assert lanes(HESSIAN, 48, 12000) == 8
     assert lanes(SDDMM_DIAG, 32, 10000) == 4 and lanes(SPMM, 48, 10000) == 8
     assert lanes(SPMM, 32, 10 ** 6) == 4 and lanes(SPMM, 48, 80000) == 8 and lanes(SPMM, 20, 80000) == 2

@@ -1,6 +1,7 @@
 """The FP64 operators' unit layout where test_gpu_units.py's few rows do not lead: two and four lanes per
 row, which many rows take, with every count of units per lane, odd row counts, and six and seven units
-per lane at eight lanes.  Against the oracle's definitions, FP64, 1e-12 of the terms' size."""
+per lane at eight lanes.  Against the oracle's definitions, FP64, 1e-12 of the terms' size.  And the FP32
+product with diagonal constraints."""
 import numpy as np
 import pytest
 
@@ -63,3 +64,26 @@ def test_fp64_operators(cuda, instances, kind, rows, ld):
                       (S.cpu().numpy()[:, :r], sdp.At_times(w, V) - sdp.C_times(V) + 0.75 * V)):
         assert np.abs(got - want).max() <= 1e-12 * np.abs(want).max()
     assert np.all(H.cpu().numpy()[:, r:] == 0.0) and np.all(S.cpu().numpy()[:, r:] == 0.0)
+
+
+@pytest.mark.parametrize("rows,r", [(TWO, 9), (301, 9), (301, 40), (TWO, 20), (117001, 7)])
+def test_fp32_product_with_diagonal_constraints(cuda, instances, rows, r):
+    """Rows of 1 to some 12 entries of C, eight a round with few rows and four with many."""
+    torch = cuda
+    inst, sdp = instances("er", rows)
+    ld = (r + 3) // 4 * 4
+    rng = np.random.default_rng(r)
+    V = (rng.standard_normal((sdp.n, r)) / np.sqrt(r)).astype(np.float32).astype(np.float64)
+    w = rng.standard_normal(sdp.m)
+    dV = torch.zeros((sdp.n, ld), dtype=torch.float32, device="cuda")
+    dV[:, :r] = torch.as_tensor(V)
+    S = torch.full_like(dV, float("nan"))
+    p = L.Problem(inst)
+    assert L.lorads_op_spmm(p.handle, L.LORADS_PREC_MIXED, r, ld, torch.as_tensor(w, device="cuda"),
+                            0.75, dV, S) == 0
+    got = S.cpu().numpy()
+    p.close()
+    want = sdp.At_times(w, V) - sdp.C_times(V) + 0.75 * V
+    # at most some 20 terms an element, of at most its scale each: 32 roundings
+    assert np.abs(got[:, :r] - want).max() <= 32 * 2.0 ** -24 * np.abs(want).max()
+    assert np.all(got[:, r:] == 0.0)
